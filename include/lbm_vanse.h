@@ -78,7 +78,8 @@ typedef struct {
     int strip_rows;              /* rows per CTA strip of the step kernel; 0 = automatic */
     int eager;                   /* 1 = launch each step on its own; 0 = replay runs of steady
                                     steps as a captured CUDA graph (default) */
-    int kernel;                  /* step-kernel variant: 0 = automatic; 1 = one column per thread
+    int kernel;                  /* step-kernel variant: 0 = automatic (kernel 5, or its phases on
+                                    tiles for small lattices and solid cells; 1 for FP64 and x walls); 1 = one column per thread
                                     (any storage); 2, 3, 4 = two columns per thread on packed FP32
                                     pairs with 64 / 96 / 128-thread CTAs; 5 = one warp per CTA,
                                     two columns per lane (2..5: not FP64) */
@@ -421,8 +422,10 @@ long long lbm_vanse_step_count(lbm_vanse_t h);
  * (9 populations in and out, phi, plus phi(t+1) and the force field when set). */
 double lbm_vanse_bytes_per_cell(lbm_vanse_t h);
 
-/* Launch shape of the step kernel: threads per CTA, output columns per CTA,
- * rows per strip, CTAs in x and y, dynamic shared memory bytes. Any may be NULL. */
+/* Launch shape of the lattice's marching step kernel: threads per CTA, output columns
+ * per CTA, rows per strip, CTAs in x and y, dynamic shared memory bytes. Any may be NULL.
+ * (With kernel = 0, plain steps of small lattices and of lattices with solid cells run as
+ * tiles of 60 columns by 4 or 8 rows instead, one warp per row.) */
 lbm_status lbm_vanse_launch_shape(lbm_vanse_t h, int* threads, int* cols, int* rows, int* grid_x,
                                   int* grid_y, int* smem_bytes);
 

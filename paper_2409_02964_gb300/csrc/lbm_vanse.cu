@@ -23,6 +23,7 @@
 #include "vanse_batch.cuh"
 #include "vanse_pair.cuh"
 #include "vanse_step.cuh"
+#include "vanse_tile.cuh"
 #include "vanse_warp.cuh"
 
 using namespace lbmv;
@@ -78,7 +79,15 @@ struct lbm_vanse {
     int* tile_order = nullptr;              // ... their launch order (those tiles first), and 2 counters
     int npl = 9;                  // planes per population buffer (11 with the momentum base)
     int* zero_phi = nullptr;      // device flag: the last phi upload held a zero
-    unsigned* step_ctr = nullptr; // device step count of the one-warp kernel (seeds stochastic rounding)
+    // device step count of kernel 5 (seeds stochastic rounding), one slot per population
+    // buffer: a step from buffer b reads slot b and leaves the next count in slot 1 - b
+    unsigned* step_ctr = nullptr;
+    int nsm = 1;
+    bool auto_kernel = false;     // created without asking for a kernel
+    bool tile_ok = false;         // the tile kernel may run the plain step (pick_tile)
+    int tile_rows = 0;            // output rows per CTA of the tile kernel (0: not used)
+    bool tile_big = false;        // its 12-warp instance
+    unsigned char* tile_solid = nullptr;    // its CTAs whose rows and columns hold a solid cell
     double s_nu = 0, s_e = 0;
     double scale = 1, inv_scale = 1;
     int* err = nullptr;           // device flag set by bounded waits
@@ -207,6 +216,10 @@ size_t step_smem_max(const lbm_vanse* h) {
     return (h->kernel >= 2 && h->kernel <= 5) ? b : b + (h->has_solid ? 0 : StepLayout<S, R, kThreads>::solid_bytes());
 }
 
+// the tile kernel runs the lattice's plain steps (the step sums and the moving wall stay
+// with kernel 5)
+bool runs_tile(const lbm_vanse* h) { return h->tile_rows > 0 && !h->nee_top; }
+
 int step_threads(const lbm_vanse* h) {
     if (h->kernel == 5) return 32;
     return h->kernel >= 2 ? kPairT[h->kernel - 2] : kThreads;
@@ -232,21 +245,51 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
     return (const void*)vanse_step_kernel<S, R, kThreads>;
 }
 
-// Rows per strip (CTA): strip_rows, or automatically about five waves of resident
-// CTAs (short strips cost halo rows, long ones leave SMs idle in the last wave); ten
-// on kernel 5 with solid cells, whose CTAs next to a solid take several times as long
-// as the others: shorter strips shorten the longest CTA (on the 4096^2 channel with
-// a solid block 56 GLUPS at 24 rows against 49 at 47).
+// Rows per strip (CTA): strip_rows, or automatic. A strip of H rows steps through H + 6
+// (kernel 5: 0.9 us a row with one warp or eight per SM), so few waves of tall strips cost
+// fewer halo rows, while several waves of short ones keep the memory busier and end more
+// evenly. Kernel 5 takes the fewest waves w whose strips stay within kWaveRows[w]; FP32
+// step on one GB300 in us, strips of 1 / 2 / 3 / 5 waves: 800^2 16.2 / 19.8 / 22.8 / -,
+// 1531 x 1024 30.0 / 30.4 / 36.1 / 40, 1800 x 1400 42.4 / 42.1 / 46.3 / 53.7, 2048^2
+// 72.2 / 64.9 / 66.4 / 72.6, 3000 x 2500 119 / 105.7 / 104.2 / 110.1, 4001 x 3001
+// 185.9 / 165.8 / 164.4 / 164.2 (five waves of at least 16 rows, the rule before: 21.5,
+// 36.1, 48.1, 72.9, 110.2, 170.1). With solid cells kernel 5 cuts ten waves of at least 16
+// rows: the CTAs next to a solid take several times as long as the others, and shorter
+// strips shorten the longest CTA. The other kernels: five waves of at least 16 rows.
 void pick_strip_height(lbm_vanse* h) {
+    static const int kWaveRows[4] = {24, 36, 40, 44};
     int H = h->prm.strip_rows;
-    if (H <= 0) {
+    auto rows = [&](int waves) {
+        const int nstrips = std::max(1, waves * h->resident / h->gridx);
+        return (h->prm.ny + nstrips - 1) / nstrips;
+    };
+    if (H <= 0 && h->kernel == 5 && !h->has_solid) {
+        int w = 1;
+        while (w < 5 && rows(w) > kWaveRows[w - 1]) ++w;
+        H = rows(w);
+    } else if (H <= 0) {
         const int waves = (h->has_solid && h->kernel == 5) ? 10 : 5;
         const int nstrips = std::max(1, (waves * h->resident + h->gridx - 1) / h->gridx);
-        H = (h->prm.ny + nstrips - 1) / nstrips;
-        H = std::max(H, 16);
+        H = std::max((h->prm.ny + nstrips - 1) / nstrips, 16);
     }
     h->H = std::min(H, h->prm.ny);
     h->gridy = (h->prm.ny + h->H - 1) / h->H;
+}
+
+// The tile kernel (vanse_tile.cuh) instead of kernel 5, for lattices that did not ask for
+// a kernel or a strip height: small ones, where a strip's serial rows are the step's time,
+// and every one with solid cells, whose marching strips are as slow as their slowest row.
+// Rows per CTA and instance: R = 4 without spills while all CTAs fit at once (two per
+// SM), R = 4 of the 80-register instance while three per SM hold them, else R = 8. Without
+// solid cells up to two waves of the last (512^2 9.7 us against 11.1 for the marching
+// kernel in strips of 4 rows, 640^2 12.8 against 11.9).
+void pick_tile(lbm_vanse* h) {
+    const int nsm = h->nsm;
+    auto ctas = [&](int R) { return (long long)h->gridx * ((h->prm.ny + R - 1) / R); };
+    h->tile_rows = 0;
+    if (!h->has_solid && ctas(8) > 4LL * nsm) return;
+    h->tile_big = ctas(4) > 2LL * nsm;
+    h->tile_rows = ctas(4) <= 3LL * nsm ? 4 : 8;
 }
 
 template <typename S>
@@ -266,7 +309,14 @@ lbm_status configure(lbm_vanse* h) {
     CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, s1));
     CK(h, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device));
     h->resident = std::max(1, per_sm * nsm);
+    h->nsm = nsm;
     pick_strip_height(h);
+    if constexpr (!std::is_same<S, double>::value) {
+        if (h->auto_kernel && h->kernel == 5 && h->prm.eq_order != 2 && !h->jbase && h->prm.strip_rows == 0) {
+            h->tile_ok = true;
+            pick_tile(h);
+        }
+    }
     return LBM_OK;
 }
 
@@ -296,6 +346,9 @@ lbm_status configure_nee(lbm_vanse* h) {
     return LBM_OK;
 }
 
+template <typename S>
+lbm_status enqueue_ghosts(lbm_vanse* h, const StepParams<float>& p, cudaStream_t stream);
+
 // Kernel 1 with solid cells: a variant of its own (the neighbour-by-neighbour stencil
 // and the 3-row rings stay out of the other kernels); shared-memory attributes set on
 // first use.
@@ -310,12 +363,7 @@ lbm_status launch_solid_step(lbm_vanse* h, const StepParams<typename Prec<S>::R>
                 h->solid_configured = true;
             }
             CK(h, warp_solid_launch<S>(p, grid, smem, stream, sums, p.eq2 != 0));
-            // the one-warp kernel writes columns 0 .. nx-1 only
-            const long long ng = (long long)h->npl * h->prm.ny * 2 * kGhost;
-            ghost_fill_kernel<S><<<(int)std::min<long long>((ng + 255) / 256, 4096), 256, 0, stream>>>(
-                (S*)p.dst, h->plane, h->prm.nx, h->prm.ny, h->P, h->step_ctr, h->npl);
-            CK(h, cudaGetLastError());
-            return LBM_OK;
+            return enqueue_ghosts<S>(h, p, stream);   // the one-warp kernel writes columns 0 .. nx-1 only
         }
     }
     if (!h->solid_configured) {
@@ -330,6 +378,16 @@ lbm_status launch_solid_step(lbm_vanse* h, const StepParams<typename Prec<S>::R>
     if (sums) vanse_step_kernel<S, R, kThreads, true, true><<<grid, kThreads, smem, stream>>>(p);
     else vanse_step_kernel<S, R, kThreads, false, true><<<grid, kThreads, smem, stream>>>(p);
     CK(h, cudaGetLastError());
+    return LBM_OK;
+}
+
+// The ghost refresh after a step of kernel 5, launched while the step's last CTAs run
+// (the kernel waits for its predecessor before it touches memory).
+template <typename S>
+lbm_status enqueue_ghosts(lbm_vanse* h, const StepParams<float>& p, cudaStream_t stream) {
+    const long long ng = (long long)h->npl * h->prm.ny * 2 * kGhost;
+    CK(h, launch_pdl(ghost_fill_kernel<S>, dim3((unsigned)std::min<long long>((ng + 255) / 256, 4096)), dim3(256), 0,
+                     stream, (S*)p.dst, h->plane, h->prm.nx, h->prm.ny, h->P, p.step_ctr, p.step_next, h->npl));
     return LBM_OK;
 }
 
@@ -390,8 +448,17 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
     p.has_solid = h->has_solid;
     p.solid_tiles = (h->has_solid && h->kernel == 5) ? h->solid_tiles : nullptr;
     p.tile_order = p.solid_tiles ? h->tile_order : nullptr;
-    p.step_ctr = h->step_ctr;
+    p.step_ctr = h->step_ctr + src;
+    p.step_next = h->step_ctr + (1 - src);
     p.wait_tries = h->wait_tries;
+    if constexpr (!std::is_same<S, double>::value) {
+        if (runs_tile(h) && !sums) {
+            p.H = h->tile_rows;
+            p.solid_tiles = h->has_solid ? h->tile_solid : nullptr;
+            CK(h, tile_launch<S>(p, h->gridx, h->has_solid, h->tile_big, stream));
+            return LBM_OK;
+        }
+    }
     if (h->kernel == 5) p.pop_map = h->pop_map[src];
     dim3 grid(h->gridx, h->gridy);
     if (h->has_solid) return launch_solid_step<S>(h, p, grid, smem, stream, sums != nullptr);
@@ -419,11 +486,7 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
                     else vanse_warp_kernel<S, LBMV_WARP_MINB, true><<<grid, 32, smem, stream>>>(p);
                 }
                 CK(h, cudaGetLastError());
-                const long long ng = (long long)h->npl * h->prm.ny * 2 * kGhost;
-                ghost_fill_kernel<S><<<(int)std::min<long long>((ng + 255) / 256, 4096), 256, 0, stream>>>(
-                    (S*)h->f[1 - src], h->plane, h->prm.nx, h->prm.ny, h->P, h->step_ctr, h->npl);
-                CK(h, cudaGetLastError());
-                return LBM_OK;
+                return enqueue_ghosts<S>(h, p, stream);
             }
         }
         vanse_step_kernel<S, R, kThreads, true><<<grid, kThreads, smem, stream>>>(p);
@@ -445,15 +508,10 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
                     CK(h, warp_nee_launch<S>(p, grid, smem, stream, false, p.eq2 != 0));
                 } else if (!h->jbase) {
                     if (p.eq2) vanse_warp_kernel<S, LBMV_WARP_MINB, false, true><<<grid, 32, smem, stream>>>(p);
-                    else vanse_warp_kernel<S, LBMV_WARP_MINB><<<grid, 32, smem, stream>>>(p);
+                    else CK(h, launch_pdl(vanse_warp_kernel<S, LBMV_WARP_MINB>, grid, dim3(32), smem, stream, p));
                 }
                 CK(h, cudaGetLastError());
-                // the one-warp kernel writes columns 0 .. nx-1 only
-                const long long ng = (long long)h->npl * h->prm.ny * 2 * kGhost;
-                ghost_fill_kernel<S><<<(int)std::min<long long>((ng + 255) / 256, 4096), 256, 0, stream>>>(
-                    (S*)h->f[1 - src], h->plane, h->prm.nx, h->prm.ny, h->P, h->step_ctr, h->npl);
-                CK(h, cudaGetLastError());
-                return LBM_OK;
+                return enqueue_ghosts<S>(h, p, stream);   // the one-warp kernel writes columns 0 .. nx-1 only
             }
             default: break;
         }
@@ -518,6 +576,14 @@ lbm_status replay_graph(lbm_vanse* h) {
 cudaError_t zero_j_planes(lbm_vanse* h, int b) {
     return cudaMemsetAsync((char*)h->f[b] + (size_t)9 * h->plane * h->sbytes, 0, (size_t)2 * h->plane * h->sbytes,
                            h->stream);
+}
+
+// New populations go to buffer 0; the step count moves with them.
+lbm_status to_buffer0(lbm_vanse* h) {
+    if (h->cur != 0)
+        CK(h, cudaMemcpyAsync(h->step_ctr, h->step_ctr + 1, sizeof(unsigned), cudaMemcpyDeviceToDevice, h->stream));
+    h->cur = 0;
+    return LBM_OK;
 }
 
 template <typename S>
@@ -731,6 +797,14 @@ lbm_status update_solid_tiles(lbm_vanse* h) {
         (const float*)h->phi, h->unsteady ? (const float*)h->phin : nullptr, h->solid_tiles, h->prm.nx, h->prm.ny, h->P,
         h->W, h->H, h->prm.bc_y == LBM_BC_BOUNCEBACK);
     CK(h, cudaGetLastError());
+    if (h->tile_rows > 0) {
+        const int gy = (h->prm.ny + h->tile_rows - 1) / h->tile_rows;
+        if (!h->tile_solid) CK(h, cudaMallocAsync((void**)&h->tile_solid, (size_t)h->gridx * gy, h->stream));
+        solid_tiles_kernel<float><<<dim3(h->gridx, gy), 256, 0, h->stream>>>(
+            (const float*)h->phi, h->unsteady ? (const float*)h->phin : nullptr, h->tile_solid, h->prm.nx, h->prm.ny,
+            h->P, h->W, h->tile_rows, h->prm.bc_y == LBM_BC_BOUNCEBACK);
+        CK(h, cudaGetLastError());
+    }
     CK(h, cudaMemsetAsync(h->tile_order + nt, 0, 2 * sizeof(int), h->stream));
     solid_order_kernel<<<(nt + 255) / 256, 256, 0, h->stream>>>(h->solid_tiles, nt, h->tile_order, h->tile_order + nt);
     CK(h, cudaGetLastError());
@@ -1017,6 +1091,7 @@ extern "C" lbm_status lbm_vanse_create(const lbm_vanse_params* p, void* cuda_str
     if (h->prm.eq_order == 0) h->prm.eq_order = 3;
     h->kernel = p->kernel ? p->kernel
                           : ((p->storage == LBM_FP64 || p->bc_x == LBM_BC_BOUNCEBACK) ? 1 : kDefaultKernel);
+    h->auto_kernel = p->kernel == 0;
     h->jbase = p->dev_base == LBM_BASE_MOMENTUM;   // (checked above)
     h->npl = h->jbase ? 11 : 9;
     h->pair = h->kernel >= 2;
@@ -1037,7 +1112,7 @@ extern "C" lbm_status lbm_vanse_create(const lbm_vanse_params* p, void* cuda_str
     const size_t fldb = (size_t)h->plane * h->rbytes;
     bool ok = alloc(&h->f[0], popb) && alloc(&h->f[1], popb) && alloc(&h->phi, fldb) && alloc(&h->phin, fldb) &&
               alloc((void**)&h->err, sizeof(int)) && alloc((void**)&h->zero_phi, sizeof(int)) &&
-              alloc((void**)&h->step_ctr, sizeof(unsigned)) &&
+              alloc((void**)&h->step_ctr, 2 * sizeof(unsigned)) &&
               alloc((void**)&h->partial, kReduceBlocks * 3 * sizeof(double)) &&
               alloc((void**)&h->red_out, 4 * sizeof(double));
     if (ok) st = DISPATCH(h, configure);
@@ -1121,6 +1196,17 @@ extern "C" lbm_status lbm_vanse_set_solid_cells(lbm_vanse_t h, int enable) {
             if (h->solid_tiles) { cudaFreeAsync(h->solid_tiles, h->stream); h->solid_tiles = nullptr; }
             if (h->tile_order) { cudaFreeAsync(h->tile_order, h->stream); h->tile_order = nullptr; }
         }
+        if (h->tile_ok) {
+            const int rows = h->tile_rows;
+            pick_tile(h);
+            CK(h, h->prm.storage == LBM_FP32   ? tile_configure<float>()
+                  : h->prm.storage == LBM_FP16 ? tile_configure<__half>()
+                                               : tile_configure<__nv_bfloat16>());
+            if (h->tile_rows != rows && h->tile_solid) {
+                cudaFreeAsync(h->tile_solid, h->stream);
+                h->tile_solid = nullptr;
+            }
+        }
     }
     return update_solid_tiles(h);
 }
@@ -1165,7 +1251,8 @@ extern "C" lbm_status lbm_vanse_init_fields(lbm_vanse_t h, const double* rho, co
     if (st != LBM_OK) return st;
     st = stage_in(h, uy, n, on_device, &dy, &o3);
     if (st != LBM_OK) return st;
-    h->cur = 0;
+    st = to_buffer0(h);
+    if (st != LBM_OK) return st;
     st = DISPATCH(h, run_init, dr, dx, dy);
     if (o1) cudaFreeAsync(dr, h->stream);
     if (o2) cudaFreeAsync(dx, h->stream);
@@ -1252,7 +1339,8 @@ extern "C" lbm_status lbm_vanse_set_populations(lbm_vanse_t h, const double* f, 
     bool owned = false;
     lbm_status st = stage_in(h, f, n9, on_device, &d, &owned);
     if (st != LBM_OK) return st;
-    h->cur = 0;
+    st = to_buffer0(h);
+    if (st != LBM_OK) return st;
     st = DISPATCH(h, run_set, d);
     if (owned) cudaFreeAsync(d, h->stream);
     if (st != LBM_OK) return st;
@@ -1304,7 +1392,7 @@ extern "C" lbm_status lbm_vanse_save_state(lbm_vanse_t h, void* buf, int on_devi
     hd.drag[0] = h->drag_d0; hd.drag[1] = h->drag_d1; hd.drag[2] = h->us_x; hd.drag[3] = h->us_y;
     hd.uw[0] = h->uw_x; hd.uw[1] = h->uw_y;
     hd.dev_base = h->jbase ? 1 : 0;
-    CK(h, cudaMemcpyAsync(&hd.step_ctr, h->step_ctr, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaMemcpyAsync(&hd.step_ctr, h->step_ctr + h->cur, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     char* out = static_cast<char*>(buf);
     const cudaMemcpyKind hk = on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost;
@@ -1351,7 +1439,7 @@ extern "C" lbm_status lbm_vanse_load_state(lbm_vanse_t h, const void* buf, int o
     off += fld;
     if (hd.unsteady) { CK(h, cudaMemcpyAsync(h->phin, in + off, fld, dk, h->stream)); off += fld; }
     if (hd.has_fb) CK(h, cudaMemcpyAsync(h->fb, in + off, 2 * fld, dk, h->stream));
-    CK(h, cudaMemcpyAsync(h->step_ctr, &hd.step_ctr, sizeof(unsigned), cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaMemcpyAsync(h->step_ctr + h->cur, &hd.step_ctr, sizeof(unsigned), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     h->unsteady = hd.unsteady != 0;
     h->has_fb = hd.has_fb != 0;
@@ -1499,7 +1587,7 @@ extern "C" void lbm_vanse_destroy(lbm_vanse_t h) {
     }
     void* ptrs[] = {h->f[0], h->f[1], h->phi, h->phin, h->fb, h->err, h->partial, h->red_out, h->scratch,
                     h->staging[0], h->staging[1], h->zero_phi, h->step_ctr, h->bad_phi, h->solid_tiles,
-                    h->tile_order};
+                    h->tile_order, h->tile_solid};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (h->bad_phi_host) cudaFreeHost(h->bad_phi_host);

@@ -64,16 +64,19 @@ __device__ __forceinline__ void fill_ghosts(S* __restrict__ buf, long long plane
     row[g] = row[sx];
 }
 
-// step_ctr (optional): the one-warp kernel's step count, advanced here once per step
-// (it seeds the stochastic rounding of FP16/BF16 stores).
+// step_ctr, step_next: the one-warp kernel's step count (it seeds the stochastic
+// rounding of FP16/BF16 stores) and where the next step's goes.
 // npl: the planes of the buffer (9 populations, 11 with the momentum base's J planes).
 template <typename S>
 __global__ void ghost_fill_kernel(S* __restrict__ buf, long long plane, int nx, int ny, int P,
-                                  unsigned* __restrict__ step_ctr = nullptr, int npl = 9) {
+                                  const unsigned* __restrict__ step_ctr, unsigned* __restrict__ step_next,
+                                  int npl = 9) {
+    pdl_wait();
+    pdl_next();
     const long long n = (long long)npl * ny * 2 * kGhost;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
         fill_ghosts<S>(buf, plane, nx, ny, P, k);
-    if (step_ctr && blockIdx.x == 0 && threadIdx.x == 0) *step_ctr += 1u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *step_next = *step_ctr + 1u;
 }
 
 // Solid-cell tiles of the one-warp kernel: per CTA (its 60 columns x0 .., its strip's

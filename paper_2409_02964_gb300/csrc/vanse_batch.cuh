@@ -69,6 +69,7 @@ struct BatchCtx {
     static constexpr bool kSolid = false;
     static constexpr bool kJB = false;
     static constexpr bool kNee = false;
+    static constexpr bool kGhosts = false;
     StepParams<float> p;       // this lattice's scalars (pointers and sizes included)
     unsigned char* smem;
     int lane, xa, sa;
@@ -94,6 +95,7 @@ struct BatchCtx {
         return reinterpret_cast<const S*>(smem + L::kPop + wslot(r) * L::kPopSlot) + sa;
     }
     __device__ __forceinline__ bool row_valid(int) const { return true; }
+    static __device__ __forceinline__ constexpr int pop_stride() { return L::WW; }
 
     __device__ __forceinline__ void row_setup(int r, PRow& st) const {
         sincospif(2.0f * (float)r / (float)p.ny, &st.sy, &st.cy);

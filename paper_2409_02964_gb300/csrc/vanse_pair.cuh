@@ -54,27 +54,51 @@ template <> struct PairIO<float> {
     __device__ static V2 un(const float* p) { return mk(p[0], p[1]); }
     __device__ static V2 dec(V2 d, V2 rest, float) { return d + rest; }
     __device__ static V2 dev(V2 d, float) { return d; }
+    using W = float2;   // a stored pair
+    __device__ static W pack(V2 v) { return v.v; }
+    __device__ static float lo(W w) { return w.x; }
+    __device__ static float hi(W w) { return w.y; }
     __device__ static void st(float* p, V2 v) { *reinterpret_cast<float2*>(p) = v.v; }
     __device__ static float enc1(float f, float rest, float) { return f - rest; }
     __device__ static V2 round_rn(V2 v) { return v; }
 };
 template <> struct PairIO<__half> {
+    using W = uint32_t;   // a stored pair
+    __device__ static W pack(V2 v) {
+        const __half2 h = __float22half2_rn(v.v);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    }
+    // stochastic rounding (the conversion's .rs mode) with 32 random bits r
+    __device__ static W pack_sr(V2 v, uint32_t r) {
+        uint32_t d;
+        asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(r));
+        return d;
+    }
+    __device__ static __half lo(W w) { return reinterpret_cast<const __half*>(&w)[0]; }
+    __device__ static __half hi(W w) { return reinterpret_cast<const __half*>(&w)[1]; }
     __device__ static V2 al(const __half* p) { return V2{__half22float2(*reinterpret_cast<const __half2*>(p))}; }
     __device__ static V2 un(const __half* p) { return V2{__half22float2(__halves2half2(p[0], p[1]))}; }
     __device__ static V2 dec(V2 d, V2 rest, float ia) { return fma2(ia, d, rest); }
     __device__ static V2 dev(V2 d, float) { return d; }   // the storage's scaled units
     __device__ static void st(__half* p, V2 v) { *reinterpret_cast<__half2*>(p) = __float22half2_rn(v.v); }
-    // stochastic rounding (the conversion's .rs mode) with 32 random bits r
-    __device__ static void st_sr(__half* p, V2 v, uint32_t r) {
-        uint32_t d;
-        asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(r));
-        *reinterpret_cast<uint32_t*>(p) = d;
-    }
     __device__ static __half enc1(float f, float rest, float s) { return __float2half_rn((f - rest) * s); }
     // a pair rounded to the storage type (to nearest) and back: stored as it is, exactly
     __device__ static V2 round_rn(V2 v) { return V2{__half22float2(__float22half2_rn(v.v))}; }
 };
 template <> struct PairIO<__nv_bfloat16> {
+    using W = uint32_t;   // a stored pair
+    __device__ static W pack(V2 v) {
+        const __nv_bfloat162 h = __float22bfloat162_rn(v.v);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    }
+    // stochastic rounding (the conversion's .rs mode) with 32 random bits r
+    __device__ static W pack_sr(V2 v, uint32_t r) {
+        uint32_t d;
+        asm("cvt.rs.satfinite.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(r));
+        return d;
+    }
+    __device__ static __nv_bfloat16 lo(W w) { return reinterpret_cast<const __nv_bfloat16*>(&w)[0]; }
+    __device__ static __nv_bfloat16 hi(W w) { return reinterpret_cast<const __nv_bfloat16*>(&w)[1]; }
     __device__ static V2 al(const __nv_bfloat16* p) {
         return V2{__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p))};
     }
@@ -83,11 +107,6 @@ template <> struct PairIO<__nv_bfloat16> {
     __device__ static V2 dev(V2 d, float) { return d; }   // the storage's scaled units
     __device__ static void st(__nv_bfloat16* p, V2 v) {
         *reinterpret_cast<__nv_bfloat162*>(p) = __float22bfloat162_rn(v.v);
-    }
-    __device__ static void st_sr(__nv_bfloat16* p, V2 v, uint32_t r) {
-        uint32_t d;
-        asm("cvt.rs.satfinite.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(r));
-        *reinterpret_cast<uint32_t*>(p) = d;
     }
     __device__ static __nv_bfloat16 enc1(float f, float rest, float s) { return __float2bfloat16_rn((f - rest) * s); }
     __device__ static V2 round_rn(V2 v) { return V2{__bfloat1622float2(__float22bfloat162_rn(v.v))}; }
@@ -113,6 +132,7 @@ struct PairLayout {
 struct PRow {
     float sy, cy;   // sin, cos of k y of this row (analytic sources only)
     V2 m[9];
+    V2 ph;             // tile kernel: phi of the row, kept from phase 1
     V2 rho;
     V2 iphi, mf, rf;   // one-warp kernel: 1/phi, the full sum f and the full rho, kept from phase 1
     V2 dr, wr;

@@ -97,7 +97,8 @@ struct StepParams {
     // the one-warp kernel collides FP16/BF16 deviations in the storage's scaled units:
     // h_* x scale, rho0 x scale and inv_scale / 3 (equal to h_*, rho0, 1/3 at scale 1)
     R hs_e, hs_eps, hs_q, hs_nu, rho0s, kp3;
-    const unsigned* step_ctr;   // one-warp kernel: steps taken (seeds the stochastic rounding), or nullptr
+    const unsigned* step_ctr;   // kernel 5: steps taken (seeds the stochastic rounding)
+    unsigned* step_next;        // ... where this step leaves the count of the next one
     uint32_t wait_tries;        // polls of a staged-row wait before it gives up (kWaitTries by default)
     // one-warp kernel: the source buffer as a tensor [9 or 11][ny][P] whose box (the
     // staged width x 1 row x all planes) stages a row's population rows in one copy

@@ -111,6 +111,7 @@ struct WarpCtx {
     // into the instances that may meet it, since even untaken it slows the general row
     // path by about 7 % (instruction-cache footprint)
     static constexpr bool kNee = NEE || SOLID || JB;
+    static constexpr bool kGhosts = false;     // ghost columns are refreshed by ghost_fill_kernel
     const StepParams<float>& p;
     unsigned char* smem;
     int lane, xa, sa;
@@ -137,6 +138,7 @@ struct WarpCtx {
     __device__ __forceinline__ bool row_valid(int r) const { return !p.wall_y || (r >= 0 && r < p.ny); }
     __device__ __forceinline__ uint32_t parity(int r) const { return (uint32_t)(((r - rlo) / kWarpSlots) & 1); }
 
+    static __device__ __forceinline__ constexpr int pop_stride() { return L::WW; }
     // the per-cell sources of the step for row r (this lane's two columns): phi(t),
     // phi(t+1) and the field part of F^B, staged with the populations
     __device__ __forceinline__ void row_setup(int, PRow&) const {}
@@ -317,7 +319,7 @@ __device__ __forceinline__ bool solid_next(uint32_t m, int col) {
 template <typename S, bool FAST, typename Ctx>
 __device__ __forceinline__ void warp_phase1(const Ctx& c, PRow& st, int r) {
     using IO = PairIO<S>;
-    constexpr int RW = WarpLayout<S>::WW;
+    const auto RW = c.pop_stride();   // elements between the population planes of a row
     const auto& p = c.p;
     c.row_setup(r, st);
     const V2 phi = c.phi2(r, st);
@@ -843,10 +845,15 @@ __device__ __forceinline__ void warp_phase3(const Ctx& c, const PRow& An, const 
             c.sums.add(2, a[5] * ins);
         }
         S* cell = reinterpret_cast<S*>(p.dst) + (long long)p3 * p.P + kPadCols + c.xa;
+        using W = typename IO::W;
+        auto put = [&](int i, W v) {
+            S* q = cell + i * p.plane;
+            if constexpr (Ctx::kGhosts) c.template store_pair<IO>(q, v);
+            else *reinterpret_cast<W*>(q) = v;
+        };
         if constexpr (sizeof(S) == 4) {
-            IO::st(cell, fo[0]);
 #pragma unroll
-            for (int i = 1; i < 9; ++i) IO::st(cell + i * p.plane, fo[i]);
+            for (int i = 0; i < 9; ++i) put(i, IO::pack(fo[i]));
         } else {
             // FP16/BF16: stochastic rounding. Round-to-nearest loses every increment
             // below half a unit of the stored deviation (a slowly forced flow then
@@ -858,10 +865,10 @@ __device__ __forceinline__ void warp_phase3(const Ctx& c, const PRow& An, const 
                                       ((c.step ^ c.salt) * 0xC2B2AE3Du));
 #pragma unroll
             for (int i = 0; i < 9; ++i)
-                IO::st_sr(cell + i * p.plane, fo[i], h0 * (0x2545F491u + 0x9E3779B8u * (uint32_t)i));
+                put(i, IO::pack_sr(fo[i], h0 * (0x2545F491u + 0x9E3779B8u * (uint32_t)i)));
             if constexpr (Ctx::kJB) {
-                IO::st(cell + 9 * p.plane, Jq);     // exact: already rounded
-                IO::st(cell + 10 * p.plane, Jqy);
+                put(9, IO::pack(Jq));     // exact: already rounded
+                put(10, IO::pack(Jqy));
             }
         }
     }
@@ -1013,6 +1020,8 @@ template <typename S, int MINB, bool SUMS = false, bool EQ2 = false, bool SOLID 
           bool NEE = false>
 __global__ void __launch_bounds__(32, MINB) vanse_warp_kernel(const __grid_constant__ StepParams<float> p) {
     extern __shared__ __align__(128) unsigned char smem[];
+    pdl_wait();
+    pdl_next();
     if constexpr (SOLID) {
         // the tiles with solid cells run first (tile_order); a CTA whose staged rows and
         // columns hold no solid cell runs the solid-free path (with its branch-free
