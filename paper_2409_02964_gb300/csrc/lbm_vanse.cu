@@ -508,7 +508,13 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
                     CK(h, warp_nee_launch<S>(p, grid, smem, stream, false, p.eq2 != 0));
                 } else if (!h->jbase) {
                     if (p.eq2) vanse_warp_kernel<S, LBMV_WARP_MINB, false, true><<<grid, 32, smem, stream>>>(p);
-                    else CK(h, launch_pdl(vanse_warp_kernel<S, LBMV_WARP_MINB>, grid, dim3(32), smem, stream, p));
+                    // early only when the strips fill the device: CTAs placed around the
+                    // predecessor's last ones otherwise pile up on some SMs (800^2, 1120 of
+                    // 1216 resident strips: 16.7 us against 15.8; 1200 x 900 24.6 / 25.3 and
+                    // 2048^2 62.8 / 66.6 the other way round)
+                    else if ((long long)h->gridx * h->gridy * 16 >= 15LL * h->resident)
+                        CK(h, launch_pdl(vanse_warp_kernel<S, LBMV_WARP_MINB>, grid, dim3(32), smem, stream, p));
+                    else vanse_warp_kernel<S, LBMV_WARP_MINB><<<grid, 32, smem, stream>>>(p);
                 }
                 CK(h, cudaGetLastError());
                 return enqueue_ghosts<S>(h, p, stream);   // the one-warp kernel writes columns 0 .. nx-1 only
