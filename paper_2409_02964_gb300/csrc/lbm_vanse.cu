@@ -216,9 +216,11 @@ size_t step_smem_max(const lbm_vanse* h) {
     return (h->kernel >= 2 && h->kernel <= 5) ? b : b + (h->has_solid ? 0 : StepLayout<S, R, kThreads>::solid_bytes());
 }
 
-// the tile kernel runs the lattice's plain steps (the step sums and the moving wall stay
-// with kernel 5)
-bool runs_tile(const lbm_vanse* h) { return h->tile_rows > 0 && !h->nee_top; }
+// a tile kernel runs the lattice's plain steps (the step sums and the moving wall stay
+// with kernel 5, and those, the moving wall and solid cells in FP64 with kernel 1)
+bool runs_tile(const lbm_vanse* h) {
+    return h->tile_rows > 0 && !h->nee_top && !(h->has_solid && h->prm.storage == LBM_FP64);
+}
 
 int step_threads(const lbm_vanse* h) {
     if (h->kernel == 5) return 32;
@@ -255,7 +257,19 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
 // 185.9 / 165.8 / 164.4 / 164.2 (five waves of at least 16 rows, the rule before: 21.5,
 // 36.1, 48.1, 72.9, 110.2, 170.1). With solid cells kernel 5 cuts ten waves of at least 16
 // rows: the CTAs next to a solid take several times as long as the others, and shorter
-// strips shorten the longest CTA. The other kernels: five waves of at least 16 rows.
+// strips shorten the longest CTA. FP64 on kernel 1: march64_us. Otherwise (kernels 1 to 4):
+// five waves of at least 16 rows.
+//
+// march64_us: a CTA (128 threads) keeps an SM's FP64 pipe 5/6 busy by itself, 7.8 us a row,
+// and two on an SM take 13 us a row; a strip of H rows steps through about H + 4. FP64
+// step in us, H = 12 / 16 / 24 / 48: 1024 x 768 380 / 472 / 365 / 406, 2000 x 1500 1317 /
+// 1400 / 1383 / 1392.
+double march64_us(const lbm_vanse* h, int H) {
+    const long long ctas = (long long)h->gridx * ((h->prm.ny + H - 1) / H), slots = 2LL * h->nsm;
+    const long long rem = ctas % slots;
+    return (H + 4) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= h->nsm ? 7.8 : 13.0)));
+}
+
 void pick_strip_height(lbm_vanse* h) {
     static const int kWaveRows[4] = {24, 36, 40, 44};
     int H = h->prm.strip_rows;
@@ -267,6 +281,10 @@ void pick_strip_height(lbm_vanse* h) {
         int w = 1;
         while (w < 5 && rows(w) > kWaveRows[w - 1]) ++w;
         H = rows(w);
+    } else if (H <= 0 && h->prm.storage == LBM_FP64 && !h->has_solid) {
+        H = 1;
+        for (int k = 2; k <= std::min(h->prm.ny, 128); ++k)
+            if (march64_us(h, k) < march64_us(h, H)) H = k;
     } else if (H <= 0) {
         const int waves = (h->has_solid && h->kernel == 5) ? 10 : 5;
         const int nstrips = std::max(1, (waves * h->resident + h->gridx - 1) / h->gridx);
@@ -290,6 +308,23 @@ void pick_tile(lbm_vanse* h) {
     if (!h->has_solid && ctas(8) > 4LL * nsm) return;
     h->tile_big = ctas(4) > 2LL * nsm;
     h->tile_rows = ctas(4) <= 3LL * nsm ? 4 : 8;
+}
+
+// The FP64 tile kernel instead of kernel 1 where it is quicker: rows per CTA by the FP64
+// pipe time of the busiest SM, CTAs per SM times kUs[R] (measured on 2000 x 1500; the same
+// figure predicts every size within 10 %). FP64 step in us, tiles / kernel 1 at 16 rows:
+// 64^2 9.6 / 137 (R = 2), 130 x 71 10 / 144 (R = 3), 256^2 40 / 145 (R = 6), 512^2 133 /
+// 246 (R = 8); 1024 x 768 398 / 365 at 24 rows.
+void pick_tile64(lbm_vanse* h) {
+    static const struct { int rows; double us; } kUs[] = {{1, 4.0}, {2, 5.8}, {3, 7.2}, {4, 8.7}, {6, 13.2}, {8, 16.6}};
+    const long long tx = (h->prm.nx + kTile64Cols - 1) / kTile64Cols;
+    double best = march64_us(h, h->H);
+    h->tile_rows = 0;
+    for (const auto& k : kUs) {
+        const long long ctas = tx * ((h->prm.ny + k.rows - 1) / k.rows);
+        const double us = k.us * (double)((ctas + h->nsm - 1) / h->nsm);
+        if (us < best) { best = us; h->tile_rows = k.rows; }
+    }
 }
 
 template <typename S>
@@ -316,6 +351,8 @@ lbm_status configure(lbm_vanse* h) {
             h->tile_ok = true;
             pick_tile(h);
         }
+    } else if (h->auto_kernel && h->prm.bc_x != LBM_BC_BOUNCEBACK && h->prm.eq_order != 2 && h->prm.strip_rows == 0) {
+        pick_tile64(h);
     }
     return LBM_OK;
 }
@@ -456,6 +493,13 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
             p.H = h->tile_rows;
             p.solid_tiles = h->has_solid ? h->tile_solid : nullptr;
             CK(h, tile_launch<S>(p, h->gridx, h->has_solid, h->tile_big, stream));
+            return LBM_OK;
+        }
+    }
+    if constexpr (std::is_same<S, double>::value) {
+        if (runs_tile(h) && !sums) {
+            p.H = h->tile_rows;
+            CK(h, tile64_launch(p, stream));
             return LBM_OK;
         }
     }
@@ -1194,6 +1238,7 @@ extern "C" lbm_status lbm_vanse_set_solid_cells(lbm_vanse_t h, int enable) {
         return fail(h, LBM_ERR_ARG, "solid cells and the momentum base together are not supported");
     h->has_solid = enable != 0;
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }   // the step's shared memory changes
+    if (h->kernel == 1) pick_strip_height(h);
     if (h->kernel == 5) {
         // the strip height follows (pick_strip_height); the tile flags are re-sized
         const int gy = h->gridy;

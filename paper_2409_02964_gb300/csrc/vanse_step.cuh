@@ -124,7 +124,7 @@ struct MomentSums {
 template <typename R>
 struct RowState {
     R m[9];                        // moments of the pulled populations (phase 1)
-    R rho;                         // rho (phase 1)
+    R rho, iphi;                   // rho, 1/phi (phase 1)
     R dr, wr;                      // x-difference / smoothed sum of rho (phase 2)
     R Fx, Fy, ux, uy;              // force and velocity (phase 2)
     R dAx, dBx, dBy, dDx;          // x-differences of rho u_x, u_x, u_y, phi rho u_x
@@ -133,7 +133,15 @@ struct RowState {
 };
 
 __device__ __forceinline__ float rcp_r(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rcp_r(double x) { return 1.0 / x; }
+// FP64: two Newton-Raphson steps from the approximate reciprocal instruction (4 FP64
+// operations; a correctly rounded division takes about ten, and the FP64 pipe, 2 lanes a
+// cycle and SM, is what bounds the FP64 step)
+__device__ __forceinline__ double rcp_r(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
 
 template <typename S, typename R, int T>
 struct StepCtx {
@@ -152,6 +160,7 @@ struct StepCtx {
     __device__ __forceinline__ uint64_t* bar(int r) const {
         return reinterpret_cast<uint64_t*>(smem) + (r & (kSlots - 1));
     }
+    static __device__ __forceinline__ constexpr int pop_stride() { return L::WW; }
     // this thread's element of population row 0 of the slot holding source row r
     __device__ __forceinline__ const S* pop(int r) const {
         return reinterpret_cast<const S*>(smem + L::kPop + (r & (kSlots - 1)) * L::kPopSlot) + sc;
@@ -201,10 +210,9 @@ struct StepCtx {
 };
 
 // Phase 1: pull + moments + rho for row r into st.
-template <typename S, typename R, int T, bool SOLID = false>
-__device__ __forceinline__ void phase1(const StepCtx<S, R, T>& c, RowState<R>& st, int r) {
-    using L = StepLayout<S, R, T>;
-    constexpr int RW = L::WW;  // elements between population rows of a slot
+template <typename S, typename R, bool SOLID = false, typename Ctx>
+__device__ __forceinline__ void phase1(const Ctx& c, RowState<R>& st, int r) {
+    const auto RW = c.pop_stride();  // elements between the population planes of a row
     const StepParams<R>& p = c.p;
     const R phi = *c.aux(r, 0);
     const Rest<R>& rs = p.rest;
@@ -254,6 +262,7 @@ __device__ __forceinline__ void phase1(const StepCtx<S, R, T>& c, RowState<R>& s
 #pragma unroll
             for (int k = 0; k < 9; ++k) st.m[k] = (R)0;
             st.rho = (R)0;
+            st.iphi = (R)0;
             return;
         }
         const R* ph0 = c.aux(r, 0);
@@ -288,7 +297,8 @@ __device__ __forceinline__ void phase1(const StepCtx<S, R, T>& c, RowState<R>& s
     st.m[6] = (R)-2 * d24 + dy;
     st.m[7] = a13 - a24;
     st.m[8] = b57 - b68;
-    st.rho = st.m[0] * rcp_r(phi);
+    st.iphi = rcp_r(phi);
+    st.rho = st.m[0] * st.iphi;
 }
 
 // 3-row ring index of a (possibly negative) row number
@@ -362,15 +372,17 @@ __device__ __forceinline__ bool solid_grad12(const StepParams<R>& p, int y, bool
 }
 
 // Phase 2 for row p2 (state Bs), rows p2-1 / p2+1 in Cs / An.
-template <typename S, typename R, int T, bool SOLID = false>
-__device__ __forceinline__ void phase2(const StepCtx<S, R, T>& c, const RowState<R>& An, RowState<R>& Bs,
-                                       const RowState<R>& Cs, int p2, R* fbuf, const R* rho3 = nullptr) {
+// fld receives the six fields rho u_x, rho u_y, u_x, u_y, phi rho u_x, phi rho u_y of the
+// cell. T, t, rho3: with solid cells the 3-row ring of rho (rows of T values).
+template <typename S, typename R, int T = 0, bool SOLID = false, typename Ctx>
+__device__ __forceinline__ void phase2(const Ctx& c, const RowState<R>& An, RowState<R>& Bs, const RowState<R>& Cs,
+                                       int p2, R fld[6], const R* rho3 = nullptr) {
     const StepParams<R>& p = c.p;
     const R twelfth = (R)1 / (R)12;
     if (SOLID && *c.aux(p2, 0) == (R)0) {   // solid cell: no velocity, no force, zero fields
         Bs.Fx = Bs.Fy = Bs.ux = Bs.uy = (R)0;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) fbuf[k * T + c.t] = (R)0;
+        for (int k = 0; k < 6; ++k) fld[k] = (R)0;
         return;
     }
     R dlo = Cs.dr, wlo = Cs.wr, dhi = An.dr, whi = An.wr;
@@ -415,18 +427,17 @@ __device__ __forceinline__ void phase2(const StepCtx<S, R, T>& c, const RowState
         uy = (Bs.m[5] + (R)0.5 * Fy) * inv;
     }
     Bs.Fx = Fx; Bs.Fy = Fy; Bs.ux = ux; Bs.uy = uy;
-    const int t = c.t;
-    fbuf[0 * T + t] = Bs.rho * ux;
-    fbuf[1 * T + t] = Bs.rho * uy;
-    fbuf[2 * T + t] = ux;
-    fbuf[3 * T + t] = uy;
-    fbuf[4 * T + t] = m0 * ux;
-    fbuf[5 * T + t] = m0 * uy;
+    fld[0] = Bs.rho * ux;
+    fld[1] = Bs.rho * uy;
+    fld[2] = ux;
+    fld[3] = uy;
+    fld[4] = m0 * ux;
+    fld[5] = m0 * uy;
 }
 
 // Phase 3 for row p3 (state Cs), rows p3-1 / p3+1 in An / Bs: C, collision, store.
-template <typename S, typename R, int T, bool SUMS = false, bool SOLID = false>
-__device__ __forceinline__ void phase3(const StepCtx<S, R, T>& c, const RowState<R>& An, const RowState<R>& Bs,
+template <typename S, typename R, int T = 0, bool SUMS = false, bool SOLID = false, typename Ctx>
+__device__ __forceinline__ void phase3(const Ctx& c, const RowState<R>& An, const RowState<R>& Bs,
                                        const RowState<R>& Cs, int p3, MomentSums<R>* sums = nullptr,
                                        const R* fld3 = nullptr) {
     const StepParams<R>& p = c.p;
@@ -512,14 +523,13 @@ __device__ __forceinline__ void phase3(const StepCtx<S, R, T>& c, const RowState
     const R phi = *c.aux(p3, 0);
     const R phin = p.unsteady ? *c.aux(p3, 1) : phi;
     const R rho = Cs.rho;
-    const R X = p.kappa * rcp_r(phi);
+    const R X = p.kappa * Cs.iphi;
     const R kp = p.model_b ? (p.kappa - (R)1) : (p.kappa - phi);
     const R kr = kp * rho;
     R Ca, Cb, Cc;
     if (!p.eq2) {
         // Eq. (20)
-        Ca = (-p.kappa * (xAx + yAy) + (R)2 * kr * (xBx + yBy) + ((R)3 - (R)2 * X) * (xDx + yDy)) * twelfth
-             - (R)2 * X * rho * (phin - phi);
+        Ca = (-p.kappa * (xAx + yAy) + (R)2 * kr * (xBx + yBy) + ((R)3 - (R)2 * X) * (xDx + yDy)) * twelfth;
         Cb = (-p.kappa * (xAx - yAy) + ((R)2 / (R)3) * kr * (xBx - yBy) + (xDx - yDy)) * twelfth;
         Cc = kr * (xBy + yBx) * ((R)1 / (R)36);
     } else {
@@ -545,11 +555,12 @@ __device__ __forceinline__ void phase3(const StepCtx<S, R, T>& c, const RowState
         }
         if (solid_nb) { xAy = xAy_s; yAx = yAx_s; xDy = xDy_s; yDx = yDx_s; }
         const R t3 = (R)2 / (R)3;
-        Ca = ((R)-2 * p.kappa * (xAx + yAy) + (R)2 * kr * (xBx + yBy) + ((R)4 - (R)2 * X) * (xDx + yDy)) * twelfth
-             - (R)2 * X * rho * (phin - phi);
+        Ca = ((R)-2 * p.kappa * (xAx + yAy) + (R)2 * kr * (xBx + yBy) + ((R)4 - (R)2 * X) * (xDx + yDy)) * twelfth;
         Cb = (-t3 * p.kappa * (xAx - yAy) + t3 * kr * (xBx - yBy) + t3 * (xDx - yDy)) * twelfth;
         Cc = (-p.kappa * (xAy + yAx) + kr * (xBy + yBx) + (xDy + yDx)) * ((R)1 / (R)36);
     }
+
+    if (p.unsteady) Ca -= (R)2 * X * rho * (phin - phi);
 
     // Eq. (18), (19), (16); the conserved moments map to m_0 and j + F for any s_c
     const R m0 = Cs.m[0], ux = Cs.ux, uy = Cs.uy, Fx = Cs.Fx, Fy = Cs.Fy;
@@ -701,7 +712,7 @@ __global__ void __launch_bounds__(T) vanse_step_kernel(const __grid_constant__ S
         c.wait_upto(p1 + 1);
         const bool ph1 = (p1 <= y1 + 1) && c.row_valid(p1);
         if (ph1) {
-            phase1<S, R, T, SOLID>(c, An, p1);
+            phase1<S, R, SOLID>(c, An, p1);
             // moving wall row: rho_b = rho of the fluid row below (its moments follow below)
             if (p.nee_top && p1 == p.ny - 1) An.rho = Bs.rho;
             rbuf[t] = An.rho;
@@ -722,10 +733,13 @@ __global__ void __launch_bounds__(T) vanse_step_kernel(const __grid_constant__ S
             An.wr = (R)4 * An.rho + (r + l);
         }
         if (ph2 && ph2_thread) {
-            phase2<S, R, T, SOLID>(c, An, Bs, Cs, p2, fbuf, rho3);
+            R fld[6];
+            phase2<S, R, T, SOLID>(c, An, Bs, Cs, p2, fld, rho3);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) fbuf[k * T + t] = fld[k];
             if constexpr (SOLID) {
 #pragma unroll
-                for (int k = 0; k < 6; ++k) fld3[(ring3(p2) * 6 + k) * T + t] = fbuf[k * T + t];
+                for (int k = 0; k < 6; ++k) fld3[(ring3(p2) * 6 + k) * T + t] = fld[k];
                 fld3[18 * T + ring3(p2) * T + t] = *c.aux(p2, 0);
             }
             if (p.nee_top && p1 == p.ny - 1 && ph1) nee_wall_moments(p, An, Bs, *c.aux(p1, 0), *c.aux(p2, 0));
@@ -746,15 +760,15 @@ __global__ void __launch_bounds__(T) vanse_step_kernel(const __grid_constant__ S
             Bs.dBx = Bxr - Bxl;
             Bs.dBy = Byr - Byl;
             Bs.dDx = Dxr - Dxl;
-            Bs.wAy = (R)4 * (Bs.rho * Bs.uy) + (Ayr + Ayl);
+            Bs.wAy = (R)4 * F0[1 * T] + (Ayr + Ayl);
             Bs.wBy = (R)4 * Bs.uy + (Byr + Byl);
             Bs.wBx = (R)4 * Bs.ux + (Bxr + Bxl);
-            Bs.wDy = (R)4 * (Bs.m[0] * Bs.uy) + (Dyr + Dyl);
+            Bs.wDy = (R)4 * F0[5 * T] + (Dyr + Dyl);
             if (p.eq2) {
                 Bs.dAy = Ayr - Ayl;
-                Bs.wAx = (R)4 * (Bs.rho * Bs.ux) + (Axr + Axl);
+                Bs.wAx = (R)4 * F0[0 * T] + (Axr + Axl);
                 Bs.dDy = Dyr - Dyl;
-                Bs.wDx = (R)4 * (Bs.m[0] * Bs.ux) + (Dxr + Dxl);
+                Bs.wDx = (R)4 * F0[4 * T] + (Dxr + Dxl);
             }
         }
         const bool ph3 = (p3 >= y0) && (p3 < y1);

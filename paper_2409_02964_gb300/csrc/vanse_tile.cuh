@@ -191,4 +191,41 @@ cudaError_t tile_configure();
 template <typename S>
 cudaError_t tile_launch(const StepParams<float>& p, int gridx, bool solid, bool big, cudaStream_t stream);
 
+
+// ------------------------------------------------------------------ FP64
+// The FP64 step on tiles of 28 columns x R rows: one warp per row, one column per lane, the
+// phases of vanse_step.cuh (full populations, FP64 arithmetic), on lattices without x walls,
+// solid cells, a moving wall or the App. B equilibrium. Same split as above. Bound by the
+// FP64 pipe (2 lanes a cycle and SM): R = 8 is 2180 FP64 warp operations, 16.8 us at that
+// rate against 16.6 measured, so the busiest SM's CTAs are the step's time and R follows
+// from that (pick_tile64). 64^2: 137 us (marching, 16 rows) -> 9.6 us.
+struct TileCtx64 {
+    const StepParams<double>& p;
+    int xc;
+
+    __device__ __forceinline__ int row(int r) const {
+        if (!p.wall_y) {
+            if (r < 0) { r += p.ny; if (r < 0) r = p.ny - 1 - ((-1 - r) % p.ny); }
+            else if (r >= p.ny) { r -= p.ny; if (r >= p.ny) r %= p.ny; }
+        }
+        return r;
+    }
+    __device__ __forceinline__ long long pop_stride() const { return p.plane; }
+    __device__ __forceinline__ const double* pop(int r) const {
+        return reinterpret_cast<const double*>(p.src) + (long long)row(r) * p.P + (kPadCols + xc);
+    }
+    // the rows phi, [phi(t+1)], [F^B_x, F^B_y] in the order of the marching kernel's ring
+    __device__ __forceinline__ const double* aux(int r, int k) const {
+        const double* a = p.phi;
+        if (k == 1 && p.unsteady) a = p.phin;
+        else if (k >= 1) a = p.fb + (k - (p.unsteady ? 2 : 1)) * p.plane;
+        return a + (long long)row(r) * p.P + (kPadCols + xc);
+    }
+};
+
+constexpr int kTile64Cols = 28, kTile64Rows = 8;
+constexpr size_t tile64_smem_bytes(int warps) { return (size_t)10 * warps * 32 * sizeof(double); }
+
+cudaError_t tile64_launch(const StepParams<double>& p, cudaStream_t stream);
+
 }  // namespace lbmv

@@ -82,3 +82,32 @@ def test_small_lattices_and_solid_cells_run_as_tiles(n, solid, tiles):
     lat.init_fields(np.ones((n, n)), np.zeros((n, n)), np.zeros((n, n)))
     assert _times_out(lat) is not tiles
     lat.close()
+
+
+@pytest.mark.parametrize("extra", ["plain", "moving", "drag"])
+@pytest.mark.parametrize("wall", [False, True])
+def test_fp64_tiles_match_the_marching_kernel(wall, extra):
+    """Tiles of 28 columns by 1 to 8 rows against kernel 1: the same phases in FP64, each
+    within 1e-12 D of the oracle over a few steps (test_gpu_parity.py)."""
+    import paper_2409_02964_gb300 as P
+    for nx, ny in [(1, 1), (2, 3), (28, 2), (29, 9), (57, 4), (121, 33), (250, 70), (400, 301)]:
+        rng = np.random.default_rng(nx + ny)
+        phi = rng.uniform(0.5, 1.0, size=(ny, nx))
+        u = 0.01 * rng.normal(size=(2, ny, nx))
+        fb = 1e-5 * rng.normal(size=(2, ny, nx))
+        phin = np.clip(phi + 0.005 * rng.normal(size=phi.shape), 0.4, 1.0)
+        out = []
+        for kernel in (0, 1):
+            lat = P.Lattice(nx, ny, 0.7, s_e=1.2, s_eps=1.2, s_q=1.2, bc_y="bounceback" if wall else "periodic",
+                            storage="fp64", kernel=kernel)
+            if extra == "drag":
+                lat.set_drag(1e-2, 0.1, 1e-3, 0.0)
+            lat.set_void_fraction(phi, phin if extra == "moving" else None)
+            lat.set_body_force(1e-5, -2e-5, fb if extra == "moving" else None)
+            lat.init_fields(np.ones((ny, nx)), u[0], u[1])
+            lat.step(1)
+            lat.step(36)
+            out.append(lat.get_populations().cpu().numpy())
+            lat.close()
+        D = 0.05
+        assert np.isfinite(out[0]).all() and np.abs(out[0] - out[1]).max() <= 2e-12 * D, (nx, ny)
