@@ -78,7 +78,7 @@ struct lbm_vanse {
     unsigned char* solid_tiles = nullptr;   // kernel 5 with solid cells: CTAs whose staged region holds one
     int* tile_order = nullptr;              // ... their launch order (those tiles first), and 2 counters
     int npl = 9;                  // planes per population buffer (11 with the momentum base)
-    int* zero_phi = nullptr;      // device flag: the last phi upload held a zero
+    bool phi_zero = false;        // the last phi upload held a zero
     // device step count of kernel 5 (seeds stochastic rounding), one slot per population
     // buffer: a step from buffer b reads slot b and leaves the next count in slot 1 - b
     unsigned* step_ctr = nullptr;
@@ -92,8 +92,8 @@ struct lbm_vanse {
     double scale = 1, inv_scale = 1;
     int* err = nullptr;           // device flag set by bounded waits
     uint32_t wait_tries = kWaitTries;   // polls of a staged-row wait (lowered only to test the timeout path)
-    int* bad_phi = nullptr;       // device flags of the void-fraction check (1: phi_t, 2: phi_next)
-    int* bad_phi_host = nullptr;  // pinned copy of them
+    int* bad_phi = nullptr;       // device flags and CTA count of the void-fraction check (check_phi_kernel)
+    int* bad_phi_host = nullptr;  // its verdict, pinned
     double* partial = nullptr;    // reduction partials (kReduceBlocks * 3)
     double* red_out = nullptr;    // reduction result (3)
     double* scratch = nullptr;    // 3 dense double fields (macros / error norms)
@@ -727,73 +727,79 @@ lbm_status stage_in(lbm_vanse* h, const T* src, long long count, int on_device, 
     return LBM_OK;
 }
 
-template <typename T>
-lbm_status pad_into(lbm_vanse* h, const T* dev_src, void* dst, int* zero_seen = nullptr) {
-    const int blocks = std::min(h->prm.ny, 65535);
+// dense caller planes (on the device) into padded planes of the compute type
+lbm_status pad_into(lbm_vanse* h, const double* dev_src, void* dst, int planes) {
+    const dim3 grid(std::min(h->prm.ny, 65535), planes);
     if (h->rbytes == 8)
-        pad_field_kernel<T, double><<<blocks, kAuxThreads, 0, h->stream>>>(dev_src, (double*)dst, h->prm.nx,
-                                                                           h->prm.ny, h->P, zero_seen);
+        pad_field_kernel<double, double><<<grid, kAuxThreads, 0, h->stream>>>(dev_src, (double*)dst, h->prm.nx,
+                                                                              h->prm.ny, h->P);
     else
-        pad_field_kernel<T, float><<<blocks, kAuxThreads, 0, h->stream>>>(dev_src, (float*)dst, h->prm.nx,
-                                                                          h->prm.ny, h->P, zero_seen);
+        pad_field_kernel<double, float><<<grid, kAuxThreads, 0, h->stream>>>(dev_src, (float*)dst, h->prm.nx,
+                                                                             h->prm.ny, h->P);
     CK(h, cudaGetLastError());
     return LBM_OK;
 }
 
-template <typename T, typename S>
-lbm_status rebase_pad(lbm_vanse* h, const T* dev_src) {
+// phi(t) [and phi(t+1)] into the lattice: a plain copy while no populations are stored (or
+// they are FP64, stored as they are); otherwise the copy that also keeps the populations
+// (pad_phi_kernel, REBASE).
+template <typename T, typename S, bool REBASE>
+lbm_status put_phi_as(lbm_vanse* h, const T* phi_t, const T* phi_next) {
     using R = typename Prec<S>::R;
-    const int blocks = std::min(h->prm.ny, 65535);
-    pad_phi_rebase_kernel<T, R, S><<<blocks, kAuxThreads, 0, h->stream>>>(
-        dev_src, (R*)h->phi, (S*)h->f[h->cur], h->prm.nx, h->prm.ny, h->P, (R)(h->prm.rho0 * h->scale), h->zero_phi);
+    const dim3 grid(std::min(h->prm.ny, 65535), phi_next ? 2 : 1);
+    pad_phi_kernel<T, R, S, REBASE><<<grid, kAuxThreads, 0, h->stream>>>(
+        phi_t, phi_next, (R*)h->phi, (R*)h->phin, (S*)h->f[h->cur], h->prm.nx, h->prm.ny, h->P,
+        (R)(h->prm.rho0 * h->scale));
     CK(h, cudaGetLastError());
     return LBM_OK;
 }
 
-// phi(t) into the lattice: a plain copy while no populations are stored (or they are
-// FP64, stored as they are); otherwise the copy that also keeps the populations
-// (pad_phi_rebase_kernel).
 template <typename T>
-lbm_status put_phi_t(lbm_vanse* h, const T* dev_src) {
-    if (!h->initialised || h->prm.storage == LBM_FP64) return pad_into<T>(h, dev_src, h->phi, h->zero_phi);
+lbm_status put_phi(lbm_vanse* h, const T* phi_t, const T* phi_next) {
+    if (h->prm.storage == LBM_FP64) return put_phi_as<T, double, false>(h, phi_t, phi_next);
+    if (!h->initialised) return put_phi_as<T, float, false>(h, phi_t, phi_next);
     switch (h->prm.storage) {
-        case LBM_FP32: return rebase_pad<T, float>(h, dev_src);
-        case LBM_FP16: return rebase_pad<T, __half>(h, dev_src);
-        default: return rebase_pad<T, __nv_bfloat16>(h, dev_src);
+        case LBM_FP32: return put_phi_as<T, float, true>(h, phi_t, phi_next);
+        case LBM_FP16: return put_phi_as<T, __half, true>(h, phi_t, phi_next);
+        default: return put_phi_as<T, __nv_bfloat16, true>(h, phi_t, phi_next);
     }
 }
 
-// The void-fraction check (check_phi_kernel) of the staged fields on stream s, then
-// its verdict: the flags are copied to pinned host memory and s is synchronised. A
-// bad field fails the call before anything of the lattice changes.
-lbm_status ensure_phi_check(lbm_vanse* h) {
+// The void-fraction check (check_phi_kernel) of the staged fields on stream s; its verdict
+// is in pinned host memory once s has been synchronised. A bad field fails the call before
+// anything of the lattice changes.
+lbm_status ensure_phi_check(lbm_vanse* h, cudaStream_t s) {
     if (h->bad_phi) return LBM_OK;
-    CK(h, cudaMalloc((void**)&h->bad_phi, sizeof(int)));
-    CK(h, cudaMallocHost((void**)&h->bad_phi_host, sizeof(int)));
+    if (!h->bad_phi_host) CK(h, cudaMallocHost((void**)&h->bad_phi_host, sizeof(int)));
+    int* acc = nullptr;
+    CK(h, cudaMalloc((void**)&acc, 2 * sizeof(int)));
+    const cudaError_t e = cudaMemsetAsync(acc, 0, 2 * sizeof(int), s);
+    if (e != cudaSuccess) { cudaFree(acc); return cuda_fail(h, e, "cudaMemsetAsync"); }
+    h->bad_phi = acc;
     return LBM_OK;
 }
 
 template <typename T>
 lbm_status check_phi_fields(lbm_vanse* h, const T* phi_t, const T* phi_next, cudaStream_t s) {
-    lbm_status st = ensure_phi_check(h);
+    lbm_status st = ensure_phi_check(h, s);
     if (st != LBM_OK) return st;
     const long long n = (long long)h->prm.nx * h->prm.ny;
-    const int blocks = (int)std::min<long long>((n + kAuxThreads - 1) / kAuxThreads, 2048);
-    CK(h, cudaMemsetAsync(h->bad_phi, 0, sizeof(int), s));
-    check_phi_kernel<T><<<blocks, kAuxThreads, 0, s>>>(phi_t, n, 1, h->bad_phi);
+    const dim3 grid((unsigned)std::min<long long>((n + kAuxThreads - 1) / kAuxThreads, 1024), phi_next ? 2 : 1);
+    if (h->rbytes == 8)
+        check_phi_kernel<T, double><<<grid, kAuxThreads, 0, s>>>(phi_t, phi_next, n, h->bad_phi, h->bad_phi_host);
+    else
+        check_phi_kernel<T, float><<<grid, kAuxThreads, 0, s>>>(phi_t, phi_next, n, h->bad_phi, h->bad_phi_host);
     CK(h, cudaGetLastError());
-    if (phi_next) {
-        check_phi_kernel<T><<<blocks, kAuxThreads, 0, s>>>(phi_next, n, 2, h->bad_phi);
-        CK(h, cudaGetLastError());
-    }
-    CK(h, cudaMemcpyAsync(h->bad_phi_host, h->bad_phi, sizeof(int), cudaMemcpyDeviceToHost, s));
     return LBM_OK;
 }
 
 // after the check's stream has been synchronised
 lbm_status phi_verdict(lbm_vanse* h) {
-    const int b = *h->bad_phi_host;
-    if (!b) return LBM_OK;
+    const int flags = *(volatile int*)h->bad_phi_host, b = flags & 3;
+    if (!b) {
+        h->phi_zero = (flags & 4) != 0;
+        return LBM_OK;
+    }
     return fail(h, LBM_ERR_ARG, "%s outside [0, 1] (NaN, negative or above 1); the lattice is unchanged",
                 b == 1 ? "phi_t holds values" : (b == 2 ? "phi_next holds values" : "phi_t and phi_next hold values"));
 }
@@ -826,9 +832,7 @@ lbm_status upload_void_fraction_pinned(lbm_vanse* h, const T* phi_t, const T* ph
     chk = phi_verdict(h);
     if (chk != LBM_OK) return chk;
     CK(h, cudaStreamWaitEvent(h->stream, h->copy_done, 0));
-    CK(h, cudaMemsetAsync(h->zero_phi, 0, sizeof(int), h->stream));
-    lbm_status st = put_phi_t<T>(h, (const T*)h->staging[0]);
-    if (st == LBM_OK && phi_next) st = pad_into<T>(h, (const T*)h->staging[1], h->phin, h->zero_phi);
+    lbm_status st = put_phi<T>(h, (const T*)h->staging[0], phi_next ? (const T*)h->staging[1] : nullptr);
     if (st != LBM_OK) return st;
     CK(h, cudaEventRecord(h->staging_free, h->stream));
     return LBM_OK;
@@ -889,9 +893,7 @@ lbm_status set_void_fraction_impl(lbm_vanse* h, const T* phi_t, const T* phi_nex
         st = e == cudaSuccess ? phi_verdict(h) : cuda_fail(h, e, "void fraction check");
     }
     if (st != LBM_OK) { release(); return st; }
-    CK(h, cudaMemsetAsync(h->zero_phi, 0, sizeof(int), h->stream));
-    st = put_phi_t<T>(h, d[0]);
-    if (st == LBM_OK && phi_next) st = pad_into<T>(h, d[1], h->phin, h->zero_phi);
+    st = put_phi<T>(h, d[0], d[1]);
     release();
     if (st != LBM_OK) return st;
     h->unsteady = phi_next != nullptr;
@@ -1161,7 +1163,7 @@ extern "C" lbm_status lbm_vanse_create(const lbm_vanse_params* p, void* cuda_str
     const size_t popb = (size_t)h->npl * h->plane * h->sbytes;
     const size_t fldb = (size_t)h->plane * h->rbytes;
     bool ok = alloc(&h->f[0], popb) && alloc(&h->f[1], popb) && alloc(&h->phi, fldb) && alloc(&h->phin, fldb) &&
-              alloc((void**)&h->err, sizeof(int)) && alloc((void**)&h->zero_phi, sizeof(int)) &&
+              alloc((void**)&h->err, sizeof(int)) &&
               alloc((void**)&h->step_ctr, 2 * sizeof(unsigned)) &&
               alloc((void**)&h->partial, kReduceBlocks * 3 * sizeof(double)) &&
               alloc((void**)&h->red_out, 4 * sizeof(double));
@@ -1204,8 +1206,7 @@ extern "C" lbm_status lbm_vanse_set_body_force(lbm_vanse_t h, double gx, double 
     bool owned = false;
     lbm_status st = stage_in(h, field, 2 * n, on_device, &d, &owned);
     if (st != LBM_OK) return st;
-    st = pad_into(h, d, h->fb);
-    if (st == LBM_OK) st = pad_into(h, d + n, (char*)h->fb + (size_t)h->plane * h->rbytes);
+    st = pad_into(h, d, h->fb, 2);
     if (owned) cudaFreeAsync(d, h->stream);
     if (st != LBM_OK) return st;
     h->has_fb = true;
@@ -1584,10 +1585,8 @@ extern "C" lbm_status lbm_vanse_sync(lbm_vanse_t h) {
     int flag = 0;
     CK(h, cudaMemcpy(&flag, h->err, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag) return fail(h, LBM_ERR_TIMEOUT, "a step kernel gave up waiting for its staged rows");
-    if (!h->has_solid) {
-        CK(h, cudaMemcpy(&flag, h->zero_phi, sizeof(int), cudaMemcpyDeviceToHost));
-        if (flag) return fail(h, LBM_ERR_ARG, "phi holds zeros: solid cells need lbm_vanse_set_solid_cells (kernels 1 and 5)");
-    }
+    if (!h->has_solid && h->phi_zero)
+        return fail(h, LBM_ERR_ARG, "phi holds zeros: solid cells need lbm_vanse_set_solid_cells (kernels 1 and 5)");
     return LBM_OK;
 }
 
@@ -1637,7 +1636,7 @@ extern "C" void lbm_vanse_destroy(lbm_vanse_t h) {
         cudaEventDestroy(h->staging_free);
     }
     void* ptrs[] = {h->f[0], h->f[1], h->phi, h->phin, h->fb, h->err, h->partial, h->red_out, h->scratch,
-                    h->staging[0], h->staging[1], h->zero_phi, h->step_ctr, h->bad_phi, h->solid_tiles,
+                    h->staging[0], h->staging[1], h->step_ctr, h->bad_phi, h->solid_tiles,
                     h->tile_order, h->tile_solid};
     for (void* q : ptrs)
         if (q) cudaFree(q);

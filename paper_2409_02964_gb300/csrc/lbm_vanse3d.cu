@@ -21,8 +21,6 @@
 // value, vector components change sign).
 #include <cuda_runtime.h>
 
-#include <stdint.h>
-
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -33,6 +31,9 @@
 #include "vanse_common.cuh"
 
 namespace lbmv3 {
+
+using lbmv::rcp_nr;
+using lbmv::widen;
 
 constexpr int Q = 19;
 
@@ -180,21 +181,6 @@ __device__ __forceinline__ long long neighbour(const Geo& g, int x, int y, int z
         yn = wrapi(yn, g.ny);
     }
     return ((long long)zn * g.ny + yn) * g.nx + xn;
-}
-
-// 1 / a by Newton-Raphson from the approximate reciprocal instruction: two steps in FP64,
-// one in FP32 (a correctly rounded division costs about ten FP64 operations, and the FP64
-// pipe is what bounds the FP64 step)
-__device__ __forceinline__ double rcp_nr(double a) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    r = fma(r, fma(-a, r, 1.0), r);
-    return fma(r, fma(-a, r, 1.0), r);
-}
-__device__ __forceinline__ float rcp_nr(float a) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-    return fmaf(r, fmaf(-a, r, 1.0f), r);
 }
 
 template <typename T>
@@ -638,17 +624,6 @@ __global__ void v3_force(const T* __restrict__ rho, const T* __restrict__ phi, c
     }
     const T ph = phi[c], G[3] = {gx, gy, gz};
     for (int a = 0; a < 3; ++a) F[a * g.N + c] = (kappa - ph) / (T)3 * gr[a] + ph * G[a] + (fb ? fb[a * g.N + c] : (T)0);
-}
-
-// (double)v, exactly: a normal float's bits are moved by integer operations, since the
-// conversion instruction runs at the FP64 rate (2 lanes a cycle and SM) and there is one
-// for each of the 19 values of a cell that are read back
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) {
-    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
-    if (m == 0u) return __hiloint2double((int)b, 0);
-    if (m < 0x00800000u || m >= 0x7f800000u) return (double)v;   // subnormal, infinity, NaN
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
 // populations to / from the caller's f: out = in + sign * f_i^rest, in FP64; blockIdx.y = i

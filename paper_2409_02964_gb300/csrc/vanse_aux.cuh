@@ -117,64 +117,80 @@ __global__ void solid_order_kernel(const unsigned char* __restrict__ tiles, int 
     }
 }
 
-// Void-fraction check of a dense field before it replaces the lattice's: every value
-// must lie in [0, 1]; NaN fails. (Zeros are solid cells: without solid cells enabled
-// they are reported later, by the sync-time check of pad_field_kernel's flag.) Sets
-// the bit `which` of *bad when any value fails; block size a multiple of 32.
-template <typename T>
-__global__ void check_phi_kernel(const T* __restrict__ src, long long n, int which, int* __restrict__ bad) {
-    bool ok = true;
+// Void-fraction check of the dense fields phi(t) and (blockIdx.y = 1) phi(t+1) before they
+// replace the lattice's, in one launch: every value must lie in [0, 1]; NaN fails. (Zeros
+// are solid cells: without solid cells enabled they are reported by the next sync.) acc[0]
+// collects the bits 1 and 2 (a field fails) and 4 (a value that is zero in the compute type
+// R); the last CTA hands them to *verdict (pinned host memory) and clears acc for the next
+// call. Block size a multiple of 32.
+template <typename T, typename R>
+__global__ void check_phi_kernel(const T* __restrict__ phi_t, const T* __restrict__ phi_next, long long n,
+                                 int* __restrict__ acc, volatile int* __restrict__ verdict) {
+    const T* src = blockIdx.y ? phi_next : phi_t;
+    bool ok = true, zero = false;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const T v = src[k];
         ok = ok && v >= (T)0 && v <= (T)1;
+        zero = zero || (R)v == (R)0;
     }
-    if (!__all_sync(0xffffffffu, ok) && (threadIdx.x & 31) == 0) atomicOr(bad, which);
+    const int bits = (__syncthreads_or(!ok) ? (blockIdx.y ? 2 : 1) : 0) | (__syncthreads_or(zero) ? 4 : 0);
+    if (threadIdx.x != 0) return;
+    if (bits) atomicOr(acc, bits);
+    __threadfence();
+    if (atomicAdd(acc + 1, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+        __threadfence();
+        *verdict = atomicExch(acc, 0);
+        acc[1] = 0;
+        __threadfence_system();
+    }
 }
 
-// Copy a dense [ny][nx] field (double or float) into a padded R field (with
-// ghosts). Rows are dealt to blocks and columns to threads (32-bit indices).
-// zero_seen (optional): set to 1 when a value is exactly zero (a solid cell in phi).
+// Copy dense [ny][nx] fields (double or float) into padded R planes (with ghosts); plane
+// blockIdx.y of the source and the destination. Rows are dealt to blocks and columns to
+// threads (32-bit indices).
 template <typename Tin, typename R>
-__global__ void pad_field_kernel(const Tin* __restrict__ src, R* __restrict__ dst, int nx, int ny, int P,
-                                 int* __restrict__ zero_seen = nullptr) {
-    bool zero = false;
+__global__ void pad_field_kernel(const Tin* __restrict__ src, R* __restrict__ dst, int nx, int ny, int P) {
+    src += (long long)blockIdx.y * nx * ny;
+    dst += (long long)blockIdx.y * ny * P;
     for (int y = blockIdx.x; y < ny; y += gridDim.x) {
         const Tin* row = src + (long long)y * nx;
-        for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-            const R v = (R)row[x];
-            zero = zero || v == (R)0;
-            put_with_ghosts<R>(dst, P, nx, x, y, v);
-        }
+        for (int x = threadIdx.x; x < nx; x += blockDim.x) put_with_ghosts<R>(dst, P, nx, x, y, (R)row[x]);
     }
-    if (zero_seen && zero) *zero_seen = 1;
 }
 
-// Replace phi(t) of a lattice that already holds FP32/FP16/BF16 populations. Those
-// store f_0 as a deviation from the rest value (phi - 5 kappa / 9) rho0 of the
-// lattice's current phi, so where phi changes the stored deviation moves by
-// (phi_old - phi_new) rho0 (times the storage scale) and the populations themselves
-// stay as they are, as with FP64 storage. Cells whose phi is unchanged are not
-// written. Each thread reads only its interior cell and writes that cell and its
-// ghost images.
-template <typename Tin, typename R, typename S>
-__global__ void pad_phi_rebase_kernel(const Tin* __restrict__ src, R* __restrict__ phi, S* __restrict__ plane0,
-                                      int nx, int ny, int P, R rho0_scaled, int* __restrict__ zero_seen) {
-    bool zero = false;
+// phi(t) and (blockIdx.y = 1) phi(t+1) into the lattice's padded fields, in one launch.
+// REBASE: the lattice already holds FP32/FP16/BF16 populations. Those store f_0 as a
+// deviation from the rest value (phi - 5 kappa / 9) rho0 of the lattice's current phi, so
+// where phi(t) changes the stored deviation moves by (phi_old - phi_new) rho0 (times the
+// storage scale) and the populations themselves stay as they are, as with FP64 storage.
+// Cells whose phi is unchanged are not written. Each thread reads only its interior cell
+// and writes that cell and its ghost images.
+template <typename Tin, typename R, typename S, bool REBASE>
+__global__ void pad_phi_kernel(const Tin* __restrict__ phi_t, const Tin* __restrict__ phi_next, R* __restrict__ phi,
+                               R* __restrict__ phin, S* __restrict__ plane0, int nx, int ny, int P, R rho0_scaled) {
+    const bool next = blockIdx.y != 0;
+    const Tin* src = next ? phi_next : phi_t;
     for (int y = blockIdx.x; y < ny; y += gridDim.x) {
         const Tin* row = src + (long long)y * nx;
         for (int x = threadIdx.x; x < nx; x += blockDim.x) {
             const R v = (R)row[x];
-            zero = zero || v == (R)0;
-            const long long o = cell_off(P, x, y);
-            const R old = phi[o];
-            if (old != v) {
-                const R d = dec(plane0[o], (R)0, (R)1) + (old - v) * rho0_scaled;
-                put_with_ghosts<S>(plane0, P, nx, x, y, enc<S, R>(d, (R)0, (R)1));
+            if (next) {
+                put_with_ghosts<R>(phin, P, nx, x, y, v);
+                continue;
+            }
+            if constexpr (REBASE) {
+                const long long o = cell_off(P, x, y);
+                const R old = phi[o];
+                if (old != v) {
+                    const R d = dec(plane0[o], (R)0, (R)1) + (old - v) * rho0_scaled;
+                    put_with_ghosts<S>(plane0, P, nx, x, y, enc<S, R>(d, (R)0, (R)1));
+                    put_with_ghosts<R>(phi, P, nx, x, y, v);
+                }
+            } else {
                 put_with_ghosts<R>(phi, P, nx, x, y, v);
             }
         }
     }
-    if (zero_seen && zero) *zero_seen = 1;
 }
 
 // Pull the post-streaming populations of cell (x, y) from the stored planes.
@@ -212,6 +228,29 @@ __device__ __forceinline__ void pull_cell(const S* __restrict__ buf, const R* __
             f[i] += w3_of<T>(pi) * ((T)ex_of(pi) * jx + (T)ey_of(pi) * jy);
         }
     }
+}
+
+// Column and row of cell k of an nx-wide lattice (32-bit: lattices hold at most 2^31 cells,
+// and a 64-bit division per cell was a good part of the read-back kernels' time).
+__device__ __forceinline__ void cell_xy(long long k, int nx, int& x, int& y) {
+    y = (int)((unsigned)k / (unsigned)nx);
+    x = (int)((unsigned)k - (unsigned)y * (unsigned)nx);
+}
+
+// A cell whose pulls need no wrap, wall or solid handling (x wraps by the ghost columns).
+template <typename T>
+__device__ __forceinline__ bool plain_cell(const Lattice<T>& L, int y) {
+    return y > 0 && y < L.ny - 1 && !L.wall_x && !L.has_solid && !L.jbase;
+}
+
+// Pulled values of a plain cell as stored (scaled deviations; FP64 storage: populations),
+// widened to FP64.
+template <typename S>
+__device__ __forceinline__ void pull_stored(const S* __restrict__ buf, const Lattice<double>& L, int x, int y,
+                                            double f[9]) {
+    const S* c = buf + cell_off(L.P, x, y);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = widen(c[i * L.plane - (long long)ey_of(i) * L.P - ex_of(i)]);
 }
 
 // Store post-streaming value f_i(x, y) where the next pull will find it (the value,
@@ -283,7 +322,8 @@ __global__ void init_kernel(S* __restrict__ buf, const R* __restrict__ phi, cons
                             const double* __restrict__ uy_in, const Lattice<R> L) {
     const long long n = (long long)L.nx * L.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / L.nx), x = (int)(k % L.nx);
+        int x, y;
+        cell_xy(k, L.nx, x, y);
         const long long co = cell_off(L.P, x, y);
         const R ph = phi[co];
         if (L.has_solid && ph == (R)0) continue;   // a solid cell holds no populations
@@ -319,6 +359,11 @@ __global__ void init_kernel(S* __restrict__ buf, const R* __restrict__ phi, cons
     }
 }
 
+// Read-back kernels, 4096^2 FP32, before / after: populations 796 / 340 us, rho 1175 /
+// 500, u and p 3684 / 1010. They were bound by the FP64 pipe (a conversion and an addition
+// per population, divisions, zero products) and by 64-bit index divisions; the memory
+// traffic alone is 270, 115 and 200 us.
+//
 // Read-back and write-back of the post-streaming populations, decoded / encoded in
 // FP64 (L: the lattice's Lattice<double>): a stored deviation d reads back as
 // d / scale + f^rest with f^rest in FP64, so the value carries no rounding at the
@@ -328,9 +373,22 @@ __global__ void get_pop_kernel(const S* __restrict__ buf, const R* __restrict__ 
                                const Lattice<double> L) {
     const long long n = (long long)L.nx * L.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / L.nx), x = (int)(k % L.nx);
+        int x, y;
+        cell_xy(k, L.nx, x, y);
         double f[9];
-        pull_cell<S, R, double>(buf, phi, L, x, y, f);
+        if (plain_cell(L, y)) {
+            pull_stored(buf, L, x, y, f);
+            const double r0 = L.rest.r0(widen(phi[cell_off(L.P, x, y)]));
+            if (Prec<S>::kDev) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    const double rest = i == 0 ? r0 : L.rest.ri(i);
+                    f[i] = sizeof(S) == 4 ? f[i] + rest : fma(f[i], L.inv_scale, rest);
+                }
+            }
+        } else {
+            pull_cell<S, R, double>(buf, phi, L, x, y, f);
+        }
 #pragma unroll
         for (int i = 0; i < 9; ++i) out[i * n + k] = f[i];
     }
@@ -341,7 +399,8 @@ __global__ void set_pop_kernel(S* __restrict__ buf, const R* __restrict__ phi, c
                                const Lattice<double> L) {
     const long long n = (long long)L.nx * L.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / L.nx), x = (int)(k % L.nx);
+        int x, y;
+        cell_xy(k, L.nx, x, y);
         const double ph = (double)phi[cell_off(L.P, x, y)];
         if (L.has_solid && ph == 0.0) continue;
 #pragma unroll
@@ -358,14 +417,21 @@ __global__ void rho_kernel(const S* __restrict__ buf, const R* __restrict__ phi,
                            const Lattice<double> L) {
     const long long n = (long long)L.nx * L.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / L.nx), x = (int)(k % L.nx);
-        double f[9];
-        pull_cell<S, R, double>(buf, phi, L, x, y, f);
-        double s = 0;
+        int x, y;
+        cell_xy(k, L.nx, x, y);
+        const double ph = widen(phi[cell_off(L.P, x, y)]);
+        double f[9], s = 0;
+        if (plain_cell(L, y)) {
+            // the rest values sum to phi rho0, so one operation adds them
+            pull_stored(buf, L, x, y, f);
+            s = ((f[0] + (f[1] + f[2])) + (f[3] + f[4])) + ((f[5] + f[6]) + (f[7] + f[8]));
+            if (Prec<S>::kDev) s = fma(ph, L.rest.rho0, L.inv_scale * s);
+        } else {
+            pull_cell<S, R, double>(buf, phi, L, x, y, f);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) s += f[i];
-        const double ph = (double)phi[cell_off(L.P, x, y)];
-        rho[k] = (L.has_solid && ph == 0.0) ? 0.0 : s / ph;
+            for (int i = 0; i < 9; ++i) s += f[i];
+        }
+        rho[k] = (L.has_solid && ph == 0.0) ? 0.0 : s * rcp_nr(ph);
     }
 }
 
@@ -376,14 +442,41 @@ __global__ void vel_kernel(const S* __restrict__ buf, const R* __restrict__ phi,
                            double* __restrict__ pr, const Lattice<double> L) {
     const long long n = (long long)L.nx * L.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / L.nx), x = (int)(k % L.nx);
+        int x, y;
+        cell_xy(k, L.nx, x, y);
         const long long co = cell_off(L.P, x, y);
+        const double ph = widen(phi[co]);
+        if (plain_cell(L, y)) {
+            double f[9];
+            pull_stored(buf, L, x, y, f);
+            const double d57 = f[5] - f[7], d86 = f[8] - f[6];
+            double jx = (f[1] - f[3]) + (d57 + d86), jy = (f[2] - f[4]) + (d57 - d86);
+            if (sizeof(S) == 2) { jx *= L.inv_scale; jy *= L.inv_scale; }
+            // Eq. (10): 12 grad rho
+            const int xm = x == 0 ? L.nx - 1 : x - 1, xp = x == L.nx - 1 ? 0 : x + 1;
+            const double *q = rho + (long long)y * L.nx, *ql = q - L.nx, *qh = q + L.nx;
+            const double r = q[x], dp = qh[xp] - ql[xm], dm = ql[xp] - qh[xm];
+            const double gx = fma(4.0, q[xp] - q[xm], dp + dm), gy = fma(4.0, qh[x] - ql[x], dp - dm);
+            const double kp = (L.model_b ? (L.kappa - 1.0) : (L.kappa - ph)) * (1.0 / 36.0);
+            double Fx = fma(kp, gx, ph * L.gx), Fy = fma(kp, gy, ph * L.gy), m0 = ph * r;
+            if (fb) { Fx += widen(fb[co]); Fy += widen(fb[L.plane + co]); }
+            if (L.has_drag) {   // Eq. (7) with the drag -beta (u - u_s) inside F, solved for u
+                const double beta = drag_beta(L, ph);
+                Fx = fma(beta, L.us_x, Fx);
+                Fy = fma(beta, L.us_y, Fy);
+                m0 = fma(0.5, beta, m0);
+            }
+            const double inv = rcp_nr(m0);
+            if (ux) ux[k] = fma(0.5, Fx, jx) * inv;
+            if (uy) uy[k] = fma(0.5, Fy, jy) * inv;
+            if (pr) pr[k] = r * (1.0 / 3.0);
+            continue;
+        }
         double f[9];
         pull_cell<S, R, double>(buf, phi, L, x, y, f);
         double s = 0, jx = 0, jy = 0;
 #pragma unroll
         for (int i = 0; i < 9; ++i) { s += f[i]; jx += (double)ex_of(i) * f[i]; jy += (double)ey_of(i) * f[i]; }
-        const double ph = (double)phi[co];
         if (L.has_solid && ph == 0.0) {   // a solid cell reports zeros
             if (ux) ux[k] = 0.0;
             if (uy) uy[k] = 0.0;

@@ -339,7 +339,8 @@ __global__ void batch_init_kernel(const BatchLattice* lats, int index, float sca
     const Lattice<float> Q = batch_as_lattice(L, scale, inv_scale);
     const long long n = (long long)L.nx * L.ny;
     for (long long kk = blockIdx.x * (long long)blockDim.x + threadIdx.x; kk < n; kk += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(kk / L.nx), x = (int)(kk % L.nx);
+        int x, y;
+        cell_xy(kk, L.nx, x, y);
         float sx, cx, sy, cy;
         sincospif(2.0f * (float)x / (float)L.nx, &sx, &cx);
         sincospif(2.0f * (float)y / (float)L.ny, &sy, &cy);
@@ -378,13 +379,14 @@ __device__ __forceinline__ void batch_pull(const BatchLattice& L, const Lattice<
                                            double f[9]) {
     const S* buf = reinterpret_cast<const S*>(L.buf[t & 1]);
     const double ph = (double)batch_phi(L, x, y, cosf(L.w * (float)t));
-    const double kr = (double)L.kappa * (double)L.rho0;
+    const double kr = (double)L.kappa * (double)L.rho0, rax = kr * (1.0 / 9.0), rdg = kr * (1.0 / 36.0);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int sx = x - ex_of(i);
-        const int sy = (y - ey_of(i) + L.ny) % L.ny;
+        int sy = y - ey_of(i);
+        sy = sy < 0 ? sy + L.ny : (sy >= L.ny ? sy - L.ny : sy);
         const S v = buf[i * L.plane + cell_off(L.P, sx, sy)];
-        const double rest = i == 0 ? ph * (double)L.rho0 - kr * (5.0 / 9.0) : kr * (i <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
+        const double rest = i == 0 ? ph * (double)L.rho0 - kr * (5.0 / 9.0) : (i <= 4 ? rax : rdg);
         f[i] = decd(v, rest, (double)Q.inv_scale);
     }
 }
@@ -397,7 +399,8 @@ __global__ void batch_get_kernel(const BatchLattice* lats, int index, const int*
     const int t = *clock;
     const long long n = (long long)L.nx * L.ny;
     for (long long kk = blockIdx.x * (long long)blockDim.x + threadIdx.x; kk < n; kk += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(kk / L.nx), x = (int)(kk % L.nx);
+        int x, y;
+        cell_xy(kk, L.nx, x, y);
         double f[9];
         batch_pull<S>(L, Q, t, x, y, f);
 #pragma unroll
@@ -415,7 +418,8 @@ __global__ void batch_rho_kernel(const BatchLattice* lats, int index, const int*
     const float ct = cosf(L.w * (float)t);
     const long long n = (long long)L.nx * L.ny;
     for (long long kk = blockIdx.x * (long long)blockDim.x + threadIdx.x; kk < n; kk += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(kk / L.nx), x = (int)(kk % L.nx);
+        int x, y;
+        cell_xy(kk, L.nx, x, y);
         double f[9];
         batch_pull<S>(L, Q, t, x, y, f);
         double s = 0.0;
@@ -438,7 +442,8 @@ __global__ void batch_err_kernel(const BatchLattice* lats, int index, const int*
     const long long n = (long long)L.nx * L.ny;
     double num = 0, den = 0;
     for (long long kk = blockIdx.x * (long long)blockDim.x + threadIdx.x; kk < n; kk += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(kk / L.nx), x = (int)(kk % L.nx);
+        int x, y;
+        cell_xy(kk, L.nx, x, y);
         double f[9];
         batch_pull<S>(L, Q, t, x, y, f);
         double s = 0, jx = 0, jy = 0;

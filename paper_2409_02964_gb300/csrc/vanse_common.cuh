@@ -36,20 +36,49 @@ template <> struct Prec<__nv_bfloat16> { using R = float; static constexpr bool 
 
 template <typename R> __device__ __forceinline__ R to_r(double v) { return (R)v; }
 
+// 1 / a by Newton-Raphson from the approximate reciprocal instruction: two steps in FP64
+// (4 FP64 operations; a correctly rounded division takes about ten, and the FP64 pipe, 2
+// lanes a cycle and SM, is what bounds the FP64 kernels), one in FP32.
+__device__ __forceinline__ double rcp_nr(double a) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+    r = fma(r, fma(-a, r, 1.0), r);
+    return fma(r, fma(-a, r, 1.0), r);
+}
+__device__ __forceinline__ float rcp_nr(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return fmaf(r, fmaf(-a, r, 1.0f), r);
+}
+
 __device__ __forceinline__ double dec(double s, double, double) { return s; }
 __device__ __forceinline__ float dec(float s, float rest, float inv_scale) { return fmaf(s, inv_scale, rest); }
 __device__ __forceinline__ float dec(__half s, float rest, float inv_scale) { return fmaf(__half2float(s), inv_scale, rest); }
 __device__ __forceinline__ float dec(__nv_bfloat16 s, float rest, float inv_scale) { return fmaf(__bfloat162float(s), inv_scale, rest); }
 
+// (double)v, exactly, by integer operations (a subnormal through an FP32 multiplication by
+// 2^64): the conversion instruction runs at the FP64 rate (2 lanes a cycle and SM), predicated
+// off as well, and the read-back kernels have one for each population of a cell.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    const bool small = m < 0x00800000u;
+    const uint32_t n = small ? __float_as_uint(__uint_as_float(m) * 18446744073709551616.0f) : m;
+    uint32_t off = small ? 0x38000000u - (64u << 20) : 0x38000000u;   // exponent bias 1023 - 127 (- 64)
+    if (m >= 0x7f800000u) off = 0x70000000u;                          // infinity, NaN
+    if (m == 0u) off = 0u;
+    return __hiloint2double((int)((b & 0x80000000u) | ((n >> 3) + off)), (int)(n << 29));
+}
+__device__ __forceinline__ double widen(__half v) { return widen(__half2float(v)); }
+__device__ __forceinline__ double widen(__nv_bfloat16 v) { return widen(__bfloat162float(v)); }
+
 // The same decode in FP64 (the read-back kernels): the stored deviation and the rest
 // value are added without the FP32 rounding at the scale of f.
 __device__ __forceinline__ double decd(double s, double, double) { return s; }
-__device__ __forceinline__ double decd(float s, double rest, double inv_scale) { return fma((double)s, inv_scale, rest); }
-__device__ __forceinline__ double decd(__half s, double rest, double inv_scale) {
-    return fma((double)__half2float(s), inv_scale, rest);
-}
+__device__ __forceinline__ double decd(float s, double rest, double) { return widen(s) + rest; }   // scale 1
+__device__ __forceinline__ double decd(__half s, double rest, double inv_scale) { return fma(widen(s), inv_scale, rest); }
 __device__ __forceinline__ double decd(__nv_bfloat16 s, double rest, double inv_scale) {
-    return fma((double)__bfloat162float(s), inv_scale, rest);
+    return fma(widen(s), inv_scale, rest);
 }
 template <typename T, typename S> __device__ __forceinline__ T dec_as(S s, T rest, T inv_scale) {
     if constexpr (sizeof(T) == 8) return decd(s, rest, inv_scale);

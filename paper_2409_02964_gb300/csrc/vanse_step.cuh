@@ -133,15 +133,7 @@ struct RowState {
 };
 
 __device__ __forceinline__ float rcp_r(float x) { return __fdividef(1.0f, x); }
-// FP64: two Newton-Raphson steps from the approximate reciprocal instruction (4 FP64
-// operations; a correctly rounded division takes about ten, and the FP64 pipe, 2 lanes a
-// cycle and SM, is what bounds the FP64 step)
-__device__ __forceinline__ double rcp_r(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
-}
+__device__ __forceinline__ double rcp_r(double x) { return rcp_nr(x); }
 
 template <typename S, typename R, int T>
 struct StepCtx {
