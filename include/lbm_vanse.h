@@ -348,7 +348,10 @@ void lbm_vanse_batch_destroy(lbm_vanse_batch_t b);
  * default) the checkpoints live in pinned host memory, and inside a segment the
  * states every K2 = ceil(sqrt(K)) steps are recomputed and also kept on the host;
  * the device holds one sub-segment of K2 states (about 2 + K2 population arrays and
- * a few fields in all; every step is recomputed twice in the backward pass). With
+ * a few fields in all; every step is recomputed twice in the backward pass). Where a
+ * whole segment of K states takes at most 512 MiB the device holds that (one
+ * recomputation), and where all nsteps states do, it keeps them from the forward pass
+ * (none; the host then holds f(0) alone). With
  * dense_segments = 1 the checkpoints and a whole segment of K states stay on the
  * device (one recomputation, K + T/K population arrays). Both give bit-identical
  * results. Everything runs in FP64 on the stream given, whatever p->storage says.

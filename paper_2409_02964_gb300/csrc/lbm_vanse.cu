@@ -16,6 +16,7 @@
 #include <string>
 #include <vector>
 #include <type_traits>
+#include <utility>
 
 #include "lbm_vanse.h"
 #include "vanse_adjoint.cuh"
@@ -2080,20 +2081,25 @@ extern "C" void lbm_vanse_batch_destroy(lbm_vanse_batch_t b) {
 
 namespace {
 
+// The device arrays of one adjoint call, carved out of one stream-ordered allocation (a
+// few dozen separate ones cost a millisecond when the pool has to map fresh memory), and
+// its pinned host checkpoints.
 struct AdjBuffers {
-    std::vector<void*> held;
+    std::vector<std::pair<double**, long long>> wanted;
+    char* base = nullptr;
     long long bytes = 0;
     void* host = nullptr;         // pinned host checkpoints
     long long host_bytes = 0;
     cudaStream_t st = nullptr;
     cudaError_t err = cudaSuccess;
-    double* get(long long n) {
-        void* q = nullptr;
-        if (err == cudaSuccess) err = cudaMallocAsync(&q, (size_t)n * sizeof(double), st);
-        if (err != cudaSuccess) return nullptr;
-        held.push_back(q);
-        bytes += n * (long long)sizeof(double);
-        return (double*)q;
+    void want(double** p, long long n) {
+        wanted.push_back({p, bytes});
+        bytes += (n * (long long)sizeof(double) + 255) / 256 * 256;
+    }
+    void allocate() {
+        if (err == cudaSuccess) err = cudaMallocAsync((void**)&base, (size_t)bytes, st);
+        if (err != cudaSuccess) { base = nullptr; return; }
+        for (auto& w : wanted) *w.first = (double*)(base + w.second);
     }
     double* get_host(long long n) {
         if (err == cudaSuccess) err = cudaMallocHost(&host, (size_t)n * sizeof(double));
@@ -2102,11 +2108,13 @@ struct AdjBuffers {
         return (double*)host;
     }
     ~AdjBuffers() {
-        for (void* q : held) cudaFreeAsync(q, st);
+        if (base) cudaFreeAsync(base, st);
         cudaStreamSynchronize(st);
         if (host) cudaFreeHost(host);
     }
 };
+
+constexpr long long kAdjKeep = 512LL << 20;   // device bytes of states kept instead of recomputed
 
 struct AdjEvents {
     cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
@@ -2147,41 +2155,49 @@ extern "C" lbm_status lbm_vanse_outlet_momentum_grad(const lbm_vanse_params* p, 
     P.s_eps = p->s_eps;
     P.s_q = p->s_q;
     P.s_nu = 1.0 / p->tau_nu;
+    P.he = 1.0 - 0.5 * P.s_e; P.heps = 1.0 - 0.5 * P.s_eps; P.hq = 1.0 - 0.5 * P.s_q; P.hnu = 1.0 - 0.5 * P.s_nu;
+    P.ne = (1.0 - P.s_e) / 36; P.neps = (1.0 - P.s_eps) / 36; P.nq = (1.0 - P.s_q) / 12; P.nnu = (1.0 - P.s_nu) / 4;
+    P.te = P.s_e / 36; P.teps = P.s_eps / 36; P.tq = P.s_q / 12; P.tnu = P.s_nu / 4;
+    P.ge = P.he / 36; P.geps = P.heps / 36; P.gq = P.hq / 12; P.gnu = P.hnu / 4;
     P.x_out = a->x_out;
     const int T = a->nsteps, M = a->avg_steps, K = a->checkpoint_every;
     const int nck = (T - 1) / K + 1;
     const bool want_grad = dJdphi != nullptr;
-    // Two levels (dense_segments = 0): the checkpoints every K steps and, while a
-    // segment is processed backwards, its states every K2 steps are kept in pinned host
-    // memory; the device holds one sub-segment of K2 states. One level: checkpoints and
-    // a whole segment of K states on the device.
+    // One level (dense_segments = 1): checkpoints and a whole segment of K states on the
+    // device. Otherwise the checkpoints are in pinned host memory, and the device holds as
+    // much as fits kAdjKeep: every state after f(0) (nothing is recomputed), or a whole
+    // segment (every step recomputed once), or else sub-segments of K2 states whose first
+    // ones are kept on the host too while a segment is processed (recomputed twice).
+    // The objective alone keeps nothing.
     const bool dense = a->dense_segments != 0;
-    const int K2 = dense ? std::min(K, T) : std::max(1, (int)std::ceil(std::sqrt((double)std::min(K, T))));
+    auto fits = [&](long long states) { return states * N9 * (long long)sizeof(double) <= kAdjKeep; };
+    const bool keep_all = want_grad && !dense && fits(T - 1);
+    const bool whole = dense || fits(std::min(K, T));   // the device holds whole segments
+    const int K2 = whole ? std::min(K, T) : std::max(1, (int)std::ceil(std::sqrt((double)std::min(K, T))));
     const int nsub = (std::min(K, T) - 1) / K2 + 1;   // sub-checkpoints per segment
 
     AdjBuffers B;
     B.st = st;
-    double* d_phi = B.get(N);
-    double* fa = B.get(N9);
-    double* fb = B.get(N9);
-    double* ck = dense ? B.get((long long)nck * N9) : B.get_host((long long)(nck + (want_grad ? nsub : 0)) * N9);
-    double* ck1 = dense ? nullptr : ck + (long long)nck * N9;   // host: a segment's sub-checkpoints
+    double *d_phi, *fa, *fb, *iphi, *acc, *ck = nullptr, *seg = nullptr, *lam = nullptr, *lam2 = nullptr, *gphi = nullptr;
     adj::Fields F;
-    F.s = B.get(N); F.rho = B.get(N); F.ux = B.get(N); F.uy = B.get(N); F.Fx = B.get(N); F.Fy = B.get(N);
-    F.drx = B.get(N); F.dry = B.get(N); F.fld = B.get(6 * N);
-    double* acc = B.get(1);
-    double *seg = nullptr, *lam = nullptr, *lam2 = nullptr, *gphi = nullptr;
     adj::Adj A;
+    B.want(&d_phi, N);
+    B.want(&fa, N9);
+    B.want(&fb, N9);
+    for (double** q : {&iphi, &F.s, &F.rho, &F.ux, &F.uy, &F.Fx, &F.Fy, &F.drx, &F.dry, &F.Ax, &F.Ay, &F.Dx, &F.Dy})
+        B.want(q, N);
+    B.want(&acc, 1);
     if (want_grad) {
-        seg = B.get((long long)K2 * N9);
-        lam = B.get(N9);
-        lam2 = B.get(N9);
-        gphi = B.get(N);
-        A.lm = B.get(N9);
-        A.lux = B.get(N); A.luy = B.get(N); A.lFx = B.get(N); A.lFy = B.get(N); A.lrho = B.get(N);
-        A.lg = B.get(8 * N);
-        A.ldrx = B.get(N); A.ldry = B.get(N);
+        if (dense) B.want(&ck, (long long)nck * N9);
+        B.want(&seg, std::max(1LL, keep_all ? T - 1LL : (long long)K2) * N9);
+        for (double** q : {&lam, &lam2, &A.lm}) B.want(q, N9);
+        for (double** q : {&gphi, &A.lux, &A.luy, &A.lFx, &A.lFy, &A.lrho, &A.ldrx, &A.ldry}) B.want(q, N);
+        B.want(&A.lg, 7 * N);
     }
+    B.allocate();
+    F.iphi = iphi;
+    if (want_grad && !dense) ck = B.get_host((keep_all ? 1LL : (long long)nck + (whole ? 0 : nsub)) * N9);
+    double* ck1 = ck + (long long)nck * N9;   // host: a segment's sub-checkpoints (not whole)
     if (B.err != cudaSuccess)
         return fail(nullptr, B.err == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA,
                     "adjoint buffers (%lld device bytes, %lld host bytes): %s", B.bytes, B.host_bytes,
@@ -2193,59 +2209,78 @@ extern "C" lbm_status lbm_vanse_outlet_momentum_grad(const lbm_vanse_params* p, 
     } while (0)
     ACK(cudaMemcpyAsync(d_phi, phi, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
     ACK(cudaMemsetAsync(acc, 0, sizeof(double), st));
-    const int nb = aux_blocks(N), nt = kAuxThreads;
+    // 64-thread blocks: the FP64 pipe of the busiest SM is a kernel's time, and small blocks
+    // spread a small lattice evenly
+    constexpr int nt = 64;
+    const dim3 nb((unsigned)std::min<long long>((N + nt - 1) / nt, 1 << 22));
+    cudaError_t le = cudaSuccess;   // the first launch error
+#define ALAUNCH(kern, grid, block, ...)                                                        \
+    do {                                                                                       \
+        const cudaError_t e_ = launch_pdl(kern, grid, dim3(block), 0, st, __VA_ARGS__);        \
+        if (le == cudaSuccess) le = e_;                                                        \
+    } while (0)
     AdjEvents ev;
     for (cudaEvent_t& x : ev.e) ACK(cudaEventCreate(&x));
     cudaEvent_t e0 = ev.e[0], e1 = ev.e[1], e2 = ev.e[2];
     ACK(cudaEventRecord(e0, st));
     auto fwd_fields = [&](const double* f) {
-        adj::adj_fwd_rho<<<nb, nt, 0, st>>>(P, f, d_phi, F);
-        adj::adj_fwd_u<<<nb, nt, 0, st>>>(P, f, d_phi, F);
+        ALAUNCH(adj::adj_fwd_rho, nb, nt, P, f, F);
+        ALAUNCH(adj::adj_fwd_u, nb, nt, P, f, d_phi, F);
     };
     auto fwd_step = [&](const double* f, double* fn) {
         fwd_fields(f);
-        adj::adj_fwd_collide<<<nb, nt, 0, st>>>(P, f, d_phi, F, fn);
+        ALAUNCH(adj::adj_fwd_collide, nb, nt, P, f, d_phi, F, fn);
     };
     // forward: f(0), checkpoints every K steps, objective over the last M steps
-    adj::adj_init_kernel<<<nb, nt, 0, st>>>(P, d_phi, fa);
+    ALAUNCH(adj::adj_init_kernel, nb, nt, P, d_phi, fa, iphi);
     double *cur = fa, *nxt = fb;
+    bool have = false;   // F holds cur's fields
     const cudaMemcpyKind to_ck = dense ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     const cudaMemcpyKind from_ck = dense ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     for (int n = 0; n < T; ++n) {
-        if (n % K == 0) ACK(cudaMemcpyAsync(ck + (long long)(n / K) * N9, cur, N9 * sizeof(double), to_ck, st));
-        fwd_step(cur, nxt);
+        if (want_grad && n % K == 0 && (n == 0 || !keep_all))
+            ACK(cudaMemcpyAsync(ck + (long long)(n / K) * N9, cur, N9 * sizeof(double), to_ck, st));
+        if (keep_all && n + 1 < T) nxt = seg + (long long)n * N9;   // f(n + 1)
+        else if (keep_all) nxt = cur == fa ? fb : fa;
+        if (!have) fwd_fields(cur);
+        ALAUNCH(adj::adj_fwd_collide, nb, nt, P, cur, d_phi, F, nxt);
         std::swap(cur, nxt);
-        if (n + 1 > T - M) {
+        have = n + 1 > T - M;
+        if (have) {
             fwd_fields(cur);
-            adj::adj_objective<<<1, 256, 0, st>>>(P, cur, F, acc);
+            ALAUNCH(adj::adj_objective, dim3(1), 256, P, cur, F, acc);
         }
     }
-    ACK(cudaGetLastError());
+    ACK(le);
     ACK(cudaEventRecord(e1, st));
     double Jsum = 0.0;
     ACK(cudaMemcpyAsync(&Jsum, acc, sizeof(double), cudaMemcpyDeviceToHost, st));
     const double wgt = 1.0 / ((double)M * p->ny);
     if (want_grad) {
         ACK(cudaMemsetAsync(gphi, 0, N * sizeof(double), st));
-        // n = T: only the objective (lambda(T+1) = 0); cur holds f(T)
-        fwd_fields(cur);
-        adj::adj_bwd_collide<<<nb, nt, 0, st>>>(P, cur, d_phi, F, nullptr, A, gphi);
-        adj::adj_bwd_u<<<nb, nt, 0, st>>>(P, cur, d_phi, F, A, wgt, gphi);
-        adj::adj_bwd_rho<<<nb, nt, 0, st>>>(P, d_phi, F, A, lam, gphi);
+        // n = T: only the objective (lambda(T+1) = 0); cur holds f(T), F its fields
+        ALAUNCH(adj::adj_bwd_collide, nb, nt, P, d_phi, F, (const double*)nullptr, A, gphi);
+        ALAUNCH(adj::adj_bwd_u, nb, nt, P, d_phi, F, A, wgt, gphi);
+        ALAUNCH(adj::adj_bwd_rho, nb, nt, P, F, A, lam, gphi);
+        auto backward_step = [&](int n, const double* fn) {
+            fwd_fields(fn);
+            ALAUNCH(adj::adj_bwd_collide, nb, nt, P, d_phi, F, lam, A, gphi);
+            ALAUNCH(adj::adj_bwd_u, nb, nt, P, d_phi, F, A, n > T - M ? wgt : 0.0, gphi);
+            ALAUNCH(adj::adj_bwd_rho, nb, nt, P, F, A, lam2, gphi);
+            std::swap(lam, lam2);
+        };
         // backward over the steps m1 - 1 .. m0, whose states are seg[0 .. m1 - m0 - 1]
         auto backward = [&](int m0, int m1) {
-            for (int n = m1 - 1; n >= m0; --n) {
-                const double* fn = seg + (long long)(n - m0) * N9;
-                fwd_fields(fn);
-                adj::adj_bwd_collide<<<nb, nt, 0, st>>>(P, fn, d_phi, F, lam, A, gphi);
-                adj::adj_bwd_u<<<nb, nt, 0, st>>>(P, fn, d_phi, F, A, n > T - M ? wgt : 0.0, gphi);
-                adj::adj_bwd_rho<<<nb, nt, 0, st>>>(P, d_phi, F, A, lam2, gphi);
-                std::swap(lam, lam2);
-            }
+            for (int n = m1 - 1; n >= m0; --n) backward_step(n, seg + (long long)(n - m0) * N9);
         };
-        for (int k = nck - 1; k >= 0; --k) {
+        if (keep_all) {
+            for (int n = T - 1; n >= 1; --n) backward_step(n, seg + (long long)(n - 1) * N9);
+            ACK(cudaMemcpyAsync(fa, ck, N9 * sizeof(double), from_ck, st));
+            backward_step(0, fa);
+        }
+        for (int k = keep_all ? -1 : nck - 1; k >= 0; --k) {
             const int n0 = k * K, n1 = std::min(n0 + K, T);
-            if (dense) {
+            if (whole) {
                 ACK(cudaMemcpyAsync(seg, ck + (long long)k * N9, N9 * sizeof(double), from_ck, st));
                 for (int j = 1; j < n1 - n0; ++j) fwd_step(seg + (long long)(j - 1) * N9, seg + (long long)j * N9);
                 backward(n0, n1);
@@ -2267,8 +2302,8 @@ extern "C" lbm_status lbm_vanse_outlet_momentum_grad(const lbm_vanse_params* p, 
                 backward(m0, m1);
             }
         }
-        adj::adj_bwd_init<<<nb, nt, 0, st>>>(P, lam, gphi);
-        ACK(cudaGetLastError());
+        ALAUNCH(adj::adj_bwd_init, nb, nt, P, lam, gphi);
+        ACK(le);
         ACK(cudaMemcpyAsync(dJdphi, gphi, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     }
     ACK(cudaEventRecord(e2, st));
@@ -2283,6 +2318,7 @@ extern "C" lbm_status lbm_vanse_outlet_momentum_grad(const lbm_vanse_params* p, 
         stats->device_bytes = B.bytes;
         stats->host_bytes = B.host_bytes;
     }
+#undef ALAUNCH
 #undef ACK
     return LBM_OK;
 }
