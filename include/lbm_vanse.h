@@ -286,7 +286,7 @@ typedef struct {
     double s_e;           /* energy rate; <= 0 derives it per lattice from nu_e = nu/3 (App. A) */
     double s_eps, s_q;    /* rates shared by all lattices */
     double kappa, rho0, phi0;
-    int strip_rows;       /* rows per work unit; 0 = a default (see lbm_vanse_batch_autotune) */
+    int strip_rows;       /* most rows per work unit; 0 = automatic (see lbm_vanse_batch_autotune) */
     int eager;            /* 1 = launch every step on its own (no CUDA graph) */
 } lbm_vanse_batch_params;
 

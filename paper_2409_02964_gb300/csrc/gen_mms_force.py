@@ -48,66 +48,73 @@ def direct_force():
 # The structured evaluation: (name, kind, expression text). kind "s" = float scalar
 # (uniform per lattice and step), "v" = per-cell value of type T. Expressions use the
 # inputs sx, cx, sy, cy (T), ct, st, k, w, A, U0, phi0, nu (float) and earlier names.
+#
+# Derivatives here are with respect to kx and ky (a factor k each, restored at the end).
+# With phi tau_ij = d_j q_i + d_i q_j - u_i d_j phi - u_j d_i phi - (2/3)(div q - u . grad
+# phi) delta_ij the divergence holds no second derivative of u:
+#   div(phi tau)_x = lap q_x + (1/3) d_x div q - (7/3) u_x phi_xx - (1/3) u_y phi_xy
+#                    - ((1/3) u_x,x + div u) phi_x - (u_x,y - (2/3) u_y,x) phi_y
+# (phi_xx = phi_yy, lap q = -2 q, div q = -2 b sin sin), 53 packed operations a cell pair
+# against 170. Every line is a sum of products, each one fused operation; the first group
+# of "v" lines depends on the column only and is formed once per strip.
 STEPS = [
     # step constants
     ("a", "s", "A * ct"),                        # phi = phi0 + a sx sy
     ("b", "s", "-(A * w * st) / (2 * k)"),       # q_x = b cx sy + U0 sx cy, q_y = b sx cy - U0 cx sy
     ("bt", "s", "-(A * w * w * ct) / (2 * k)"),  # d_t b
-    ("ak", "s", "a * k"),
-    ("akk", "s", "a * k * k"),
-    ("bk", "s", "b * k"),
-    ("uk", "s", "U0 * k"),
-    ("kk", "s", "k * k"),
-    # products of the trig arguments
-    ("ss", "v", "sx * sy"),
-    ("cc", "v", "cx * cy"),
-    ("cs", "v", "cx * sy"),
-    ("sc", "v", "sx * cy"),
-    # phi and its derivatives
-    ("ph", "v", "phi0 + a * ss"),
-    ("phx", "v", "ak * cs"),
-    ("phy", "v", "ak * sc"),
-    ("phxx", "v", "-akk * ss"),                 # = phi_yy
-    ("phxy", "v", "akk * cc"),
+    ("n1", "s", "nu * k"),
+    ("c1", "s", "bt / k + (2.0 / 3.0) * n1 * b"),
+    ("c2", "s", "2 * n1"),
+    ("m7", "s", "-(7.0 / 3.0) * n1"),
+    ("m1", "s", "(1.0 / 3.0) * n1"),
+    # of the column
+    ("asx", "v", "a * sx"),
+    ("acx", "v", "a * cx"),
+    ("nasx", "v", "(-a) * sx"),
+    ("nacx", "v", "(-a) * cx"),
+    ("bsx", "v", "b * sx"),
+    ("bcx", "v", "b * cx"),
+    ("nbsx", "v", "(-b) * sx"),
+    ("usx", "v", "U0 * sx"),
+    ("ucx", "v", "U0 * cx"),
+    ("nusx", "v", "(-U0) * sx"),
+    ("nucx", "v", "(-U0) * cx"),
+    ("dsx", "v", "c1 * sx"),
+    ("dcx", "v", "c1 * cx"),
+    # phi and its derivatives (npx = -phi_x, e1 = -phi_xx = -phi_yy, e2 = phi_xy)
+    ("e1", "v", "asx * sy"),
+    ("e2", "v", "acx * cy"),
+    ("ph", "v", "asx * sy + phi0"),
+    ("npx", "v", "nacx * sy"),
+    ("npy", "v", "nasx * cy"),
     # q and its derivatives
-    ("qx", "v", "b * cs + U0 * sc"),
-    ("qy", "v", "b * sc - U0 * cs"),
-    ("qxt", "v", "bt * cs"),
-    ("qyt", "v", "bt * sc"),
-    ("qxx", "v", "uk * cc - bk * ss"),          # d_x q_x
-    ("qxy", "v", "bk * cc - uk * ss"),          # d_y q_x
-    ("qyx", "v", "bk * cc + uk * ss"),          # d_x q_y
-    ("qyy", "v", "-bk * ss - uk * cc"),         # d_y q_y
-    ("qmx", "v", "-kk * (b * sc + U0 * cs)"),   # d_x d_y q_x
-    ("qmy", "v", "kk * (U0 * sc - b * cs)"),    # d_x d_y q_y  (d_xx q = d_yy q = -k^2 q)
+    ("qx", "v", "bcx * sy + usx * cy"),
+    ("qy", "v", "bsx * cy + nucx * sy"),
+    ("nbss", "v", "nbsx * sy"),
+    ("bcc", "v", "bcx * cy"),
+    ("qxx", "v", "ucx * cy + nbss"),            # d_x q_x
+    ("qyy", "v", "nucx * cy + nbss"),           # d_y q_y
+    ("qxy", "v", "nusx * sy + bcc"),            # d_y q_x
+    ("qyx", "v", "usx * sy + bcc"),             # d_x q_y
     # u = q / phi and its derivatives (quotient rule)
     ("ip", "v", "1 / ph"),
     ("ux", "v", "qx * ip"),
     ("uy", "v", "qy * ip"),
-    ("uxx", "v", "(qxx - ux * phx) * ip"),
-    ("uxy", "v", "(qxy - ux * phy) * ip"),
-    ("uyx", "v", "(qyx - uy * phx) * ip"),
-    ("uyy", "v", "(qyy - uy * phy) * ip"),
-    ("uxXX", "v", "(-kk * qx - 2 * uxx * phx - ux * phxx) * ip"),
-    ("uxYY", "v", "(-kk * qx - 2 * uxy * phy - ux * phxx) * ip"),
-    ("uxXY", "v", "(qmx - uxx * phy - uxy * phx - ux * phxy) * ip"),
-    ("uyXX", "v", "(-kk * qy - 2 * uyx * phx - uy * phxx) * ip"),
-    ("uyYY", "v", "(-kk * qy - 2 * uyy * phy - uy * phxx) * ip"),
-    ("uyXY", "v", "(qmy - uyx * phy - uyy * phx - uy * phxy) * ip"),
-    # viscous stress and its divergence terms
+    ("uxx", "v", "(ux * npx + qxx) * ip"),
+    ("uxy", "v", "(ux * npy + qxy) * ip"),
+    ("uyx", "v", "(uy * npx + qyx) * ip"),
+    ("uyy", "v", "(uy * npy + qyy) * ip"),
     ("dv", "v", "uxx + uyy"),
-    ("txx", "v", "2 * uxx - (2.0 / 3.0) * dv"),
-    ("tyy", "v", "2 * uyy - (2.0 / 3.0) * dv"),
-    ("txy", "v", "uxy + uyx"),
-    ("dxtxx", "v", "(4.0 / 3.0) * uxXX - (2.0 / 3.0) * uyXY"),
-    ("dytyy", "v", "(4.0 / 3.0) * uyYY - (2.0 / 3.0) * uxXY"),
-    ("dytxy", "v", "uxYY + uyXY"),
-    ("dxtxy", "v", "uxXY + uyXX"),
-    ("vx", "v", "phx * txx + ph * dxtxx + phy * txy + ph * dytxy"),
-    ("vy", "v", "phx * txy + ph * dxtxy + phy * tyy + ph * dytyy"),
+    ("dc", "v", "dv + c2"),
+    ("hx", "v", "(-n1) * npx"),
+    ("hy", "v", "(-n1) * npy"),
     # Eq. (25) without the pressure term, per unit rho0
-    ("fx", "out", "qxt + qxx * ux + qx * uxx + qxy * uy + qx * uyy - nu * vx"),
-    ("fy", "out", "qyt + qyx * ux + qy * uxx + qyy * uy + qy * uyy - nu * vy"),
+    ("gx", "v", "dcx * sy + ux * (m7 * e1 + qxx) + uy * (m1 * e2 + qxy) + qx * dc"
+                " + hx * ((1.0 / 3.0) * uxx + dv) + hy * ((-2.0 / 3.0) * uyx + uxy)"),
+    ("gy", "v", "dsx * cy + uy * (m7 * e1 + qyy) + ux * (m1 * e2 + qyx) + qy * dc"
+                " + hy * ((1.0 / 3.0) * uyy + dv) + hx * ((-2.0 / 3.0) * uxy + uyx)"),
+    ("fx", "out", "k * gx"),
+    ("fy", "out", "k * gy"),
 ]
 
 INPUTS_V = ("sx", "cx", "sy", "cy")
@@ -163,8 +170,9 @@ def main() -> None:
 // phi u = grad psi + rot Psi (see the generator for the definitions), per unit rho0.
 // Arguments: sx, cx = sin, cos of k x; sy, cy = sin, cos of k y; ct, st = cos, sin
 // of w t. Evaluated from phi, q = phi u and their derivatives, u by the quotient rule.
-// T is the arithmetic type (float or a packed pair); it must provide + - * between
-// T values and with a float on either side, unary -, and mms_rcp(T).
+// T is the arithmetic type (float, or ForceV, whose products join the sum they enter in
+// one fused operation); it must provide products of T values, of a float and a T, sums of
+// these, T + float, and mms_rcp(T).
 #pragma once
 
 namespace lbmv {{

@@ -12,7 +12,9 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <functional>
 #include <numeric>
+#include <queue>
 #include <string>
 #include <vector>
 #include <type_traits>
@@ -1659,7 +1661,8 @@ struct lbm_vanse_batch {
     void* pool = nullptr;                // every population buffer
     BatchLattice* d_desc = nullptr;
     int* d_units = nullptr;              // lattice of each unit
-    int* d_clock = nullptr;              // [0] = t, [1] = unit counter, [2] = error flag
+    int* d_clock = nullptr;              // [0] = t, [1] = unit counter, [2] = error flag, [3] = ghost CTAs done
+    float2* d_trig = nullptr;            // BatchLattice::trig of every lattice
     double* scratch = nullptr;           // dense rho of the largest lattice
     double* partial = nullptr;
     double* red_out = nullptr;
@@ -1705,17 +1708,64 @@ lbm_status bfail(lbm_vanse_batch* b, lbm_status st, const char* fmt, ...) {
         }                                                                        \
     }())
 
-// Work units of height H for every lattice, largest lattices first.
+// Strips of at most H rows, of (nearly) one height: their count and that height.
+void batch_strips(int ny, int H, int* strips, int* rows) {
+    const int s = (ny + H - 1) / H;
+    *rows = (ny + s - 1) / s;
+    *strips = (ny + *rows - 1) / *rows;
+}
+
+// Rows per unit: the least time of a schedule that hands the units, highest first, to the
+// grid's CTAs as these fall free, a unit of h rows taking h + 6 row times (4 halo rows, and
+// two while its first rows are on their way). With many units per CTA the end of the
+// schedule no longer matters: the work per CTA plus one unit. us per step, this rule / 24 /
+// 48 / 96 rows: 24 lattices of 10.96 M cells FP32 188 / 203 / 196 / 185, 7 of 2.3 M 53 / 63
+// / 63 / 99, 40 of 12.6 M 202 / 232 / 213 / 202, 40 of 17.0 M BF16 267 / 296 / 274 / 278.
+int batch_rows(const lbm_vanse_batch* b) {
+    int best = 48;
+    double best_cost = 0;
+    for (int H = 12; H <= 192; H += H < 64 ? 4 : 16) {
+        std::vector<std::pair<int, long long>> kinds;   // (row times, units)
+        double sum = 0;
+        long long units = 0;
+        for (const BatchLattice& L : b->desc) {
+            int strips, rows;
+            batch_strips(L.ny, H, &strips, &rows);
+            kinds.push_back({rows + 6, (long long)L.tiles_x * strips});
+            sum += (double)(rows + 6) * L.tiles_x * strips;
+            units += (long long)L.tiles_x * strips;
+        }
+        double cost;
+        if (units > 12LL * b->grid) {
+            cost = sum / b->grid + H + 6;
+        } else {
+            std::sort(kinds.begin(), kinds.end(), std::greater<>());
+            std::priority_queue<int, std::vector<int>, std::greater<int>> free_at;
+            int end = 0;
+            for (auto& k : kinds)
+                for (long long u = 0; u < k.second; ++u) {
+                    int at = 0;
+                    if ((int)free_at.size() >= b->grid) { at = free_at.top(); free_at.pop(); }
+                    free_at.push(at + k.first);
+                    end = std::max(end, at + k.first);
+                }
+            cost = end;
+        }
+        if (best_cost == 0 || cost < best_cost) { best_cost = cost; best = H; }
+    }
+    return best;
+}
+
+// Work units of at most H rows for every lattice, the highest units first.
 lbm_status batch_decompose(lbm_vanse_batch* b, int H) {
     const int n = (int)b->lat.size();
+    for (BatchLattice& L : b->desc) batch_strips(L.ny, H, &L.strips, &L.H);
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return b->lat[a].n > b->lat[c].n; });
+    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return b->desc[a].H > b->desc[c].H; });
     std::vector<int> units;
     for (int idx : order) {
         BatchLattice& L = b->desc[idx];
-        L.H = std::min(H, L.ny);
-        L.strips = (L.ny + L.H - 1) / L.H;
         L.unit0 = (int)units.size();
         for (int u = 0; u < L.tiles_x * L.strips; ++u) units.push_back(idx);
     }
@@ -1771,12 +1821,9 @@ lbm_status batch_configure(lbm_vanse_batch* b) {
 template <typename S>
 lbm_status batch_enqueue_step(lbm_vanse_batch* b, cudaStream_t stream) {
     const size_t smem = WarpLayout<S>::bytes(0);
-    vanse_batch_kernel<S, kBatchMinBlocks><<<b->grid, 32, smem, stream>>>(batch_params(b));
-    BCK(b, cudaGetLastError());
-    batch_ghost_fill_kernel<S><<<dim3(b->ghost_blocks, (unsigned)b->desc.size()), 256, 0, stream>>>(b->d_desc, b->d_clock);
-    BCK(b, cudaGetLastError());
-    batch_tick_kernel<<<1, 1, 0, stream>>>(b->d_clock, b->d_clock + 1);
-    BCK(b, cudaGetLastError());
+    BCK(b, launch_pdl(vanse_batch_kernel<S, kBatchMinBlocks>, dim3(b->grid), dim3(32), smem, stream, batch_params(b)));
+    BCK(b, launch_pdl(batch_ghost_fill_kernel<S>, dim3(b->ghost_blocks, (unsigned)b->desc.size()), dim3(256), 0, stream,
+                      b->d_desc, b->d_clock));
     return LBM_OK;
 }
 
@@ -1830,8 +1877,6 @@ lbm_status batch_run_each(lbm_vanse_batch* b, int nsteps) {
         batch_ghost_fill_kernel<S><<<dim3(b->ghost_blocks, (unsigned)b->desc.size()), 256, 0, b->stream>>>(b->d_desc,
                                                                                                       b->d_clock);
         BCK(b, cudaGetLastError());
-        batch_tick_kernel<<<1, 1, 0, b->stream>>>(b->d_clock, b->d_clock + 1);
-        BCK(b, cudaGetLastError());
         b->steps++;
     }
     return LBM_OK;
@@ -1839,7 +1884,7 @@ lbm_status batch_run_each(lbm_vanse_batch* b, int nsteps) {
 
 template <typename S>
 lbm_status batch_do_init(lbm_vanse_batch* b) {
-    BCK(b, cudaMemsetAsync(b->d_clock, 0, 3 * sizeof(int), b->stream));
+    BCK(b, cudaMemsetAsync(b->d_clock, 0, 4 * sizeof(int), b->stream));
     for (size_t i = 0; i < b->desc.size(); ++i) {
         const long long n = (long long)b->desc[i].nx * b->desc[i].ny;
         batch_init_kernel<S><<<aux_blocks(n), kAuxThreads, 0, b->stream>>>(b->d_desc, (int)i, b->scale, b->inv_scale);
@@ -1961,7 +2006,16 @@ extern "C" lbm_status lbm_vanse_batch_create(const lbm_vanse_batch_lattice* latt
                 if (!err.empty()) st = bfail(nullptr, LBM_ERR_CUDA, "batch tensor maps: %s", err.c_str());
             }
         }
+        long long rows = 0;
+        for (auto& q : b->lat) rows += q.n;
         e = cudaMalloc((void**)&b->d_desc, count * sizeof(BatchLattice));
+        if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_trig, rows * sizeof(float2));
+        float2* tr = b->d_trig;
+        for (int i = 0; i < count && e == cudaSuccess; tr += b->lat[i].n, ++i) {
+            b->desc[i].trig = tr;
+            batch_trig_kernel<<<(b->lat[i].n + 127) / 128, 128, 0, b->stream>>>(tr, b->lat[i].n);
+            e = cudaGetLastError();
+        }
         if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_clock, 4 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_clock, 0, 4 * sizeof(int), b->stream);
         if (e == cudaSuccess) e = cudaMalloc((void**)&b->scratch, (size_t)nmax * nmax * sizeof(double));
@@ -1970,7 +2024,7 @@ extern "C" lbm_status lbm_vanse_batch_create(const lbm_vanse_batch_lattice* latt
         if (e != cudaSuccess) st = bfail(nullptr, LBM_ERR_OOM, "batch buffers: %s", cudaGetErrorString(e));
     }
     if (st == LBM_OK) st = BDISPATCH(b, batch_configure);
-    if (st == LBM_OK) st = batch_decompose(b, p->strip_rows > 0 ? p->strip_rows : 48);
+    if (st == LBM_OK) st = batch_decompose(b, p->strip_rows > 0 ? p->strip_rows : batch_rows(b));
     if (st != LBM_OK) {
         if (b->msg.size()) g_create_error = b->msg;
         lbm_vanse_batch_destroy(b);
@@ -2071,7 +2125,7 @@ extern "C" void lbm_vanse_batch_destroy(lbm_vanse_batch_t b) {
     cudaStreamSynchronize(b->stream);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    void* ptrs[] = {b->pool, b->d_desc, b->d_units, b->d_clock, b->scratch, b->partial, b->red_out};
+    void* ptrs[] = {b->pool, b->d_desc, b->d_units, b->d_clock, b->d_trig, b->scratch, b->partial, b->red_out};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete b;

@@ -53,11 +53,11 @@ __device__ __forceinline__ void put_with_ghosts(T* plane_base, int P, int nx, in
 // (a verbatim copy: an FP16 / BF16 value stays encoded against the same phi, whose
 // ghosts are images too). Runs after a step kernel that writes columns 0 .. nx-1
 // only. One thread per (plane, row, ghost column).
-template <typename S>
-__device__ __forceinline__ void fill_ghosts(S* __restrict__ buf, long long plane, int nx, int ny, int P, long long k) {
+template <typename S, typename K>
+__device__ __forceinline__ void fill_ghosts(S* __restrict__ buf, long long plane, int nx, int ny, int P, K k) {
     const int g6 = (int)(k % (2 * kGhost));
-    const long long rest = k / (2 * kGhost);
-    const int y = (int)(rest % ny), i = (int)(rest / ny);
+    const K rest = k / (2 * kGhost);
+    const int y = (int)(rest % (K)ny), i = (int)(rest / (K)ny);
     const int g = g6 < kGhost ? g6 - kGhost : nx + g6 - kGhost;
     const int sx = ((g % nx) + nx) % nx;
     S* row = buf + i * plane + (long long)y * P + kPadCols;

@@ -8,18 +8,49 @@
 // coordinates and the step count, so the step reads and writes only the
 // populations (no phi / force arrays).
 //
-// Work decomposition: every lattice is cut into units of 60 columns x H rows (the
-// one-warp kernel's tile). A persistent grid of one-warp CTAs takes units from a
-// global counter (largest lattices first) and runs the same row pipeline as the
-// single-lattice one-warp kernel (warp_run_strip). The time step t lives in device
-// memory and is advanced, with the unit counter reset, by a one-thread kernel
-// after each step, so a captured CUDA graph of (step, tick) pairs replays without
-// host involvement.
+// Work decomposition: every lattice is cut into units of 60 columns x at most H rows (the
+// one-warp kernel's tile; batch_rows picks H). A persistent grid of one-warp CTAs takes
+// units from a global counter (highest units first) and runs the same row pipeline as the
+// single-lattice one-warp kernel (warp_run_strip). The time step t lives in device memory;
+// the ghost refresh after each step advances it and resets the unit counter, so a captured
+// CUDA graph of (step, ghosts) pairs replays without host involvement, each launched
+// while its predecessor drains.
+//
+// Bound by issue and latency (two warps per scheduler, the force on top of the collision).
+// us per step, before / after the force in 53 packed operations instead of 170, tabulated
+// row sines, unit heights by schedule and one launch fewer (before: units of 48 rows): 24
+// lattices of 10.96 M cells FP32 205 / 188, FP16 214 / 179, 40 of 12.6 M FP32 260 / 202,
+// 40 of 17.0 M BF16 327 / 267, 7 of 2.3 M FP32 68.6 / 52.9.
 #pragma once
 
 #include "vanse_aux.cuh"
 #include "vanse_warp.cuh"
-// after vanse_warp.cuh: the generated code needs the pair type and mms_rcp
+
+namespace lbmv {
+
+// The pair type of the force: a product is kept as its two factors until the sum it enters
+// takes it in one fused operation (the packed intrinsics are never contracted by the
+// compiler, so V2's own operators cost an instruction each).
+struct ForceV {
+    V2 v;
+};
+struct ForceProd {
+    V2 a, b;
+    __device__ __forceinline__ operator ForceV() const { return ForceV{a * b}; }
+};
+__device__ __forceinline__ ForceProd operator*(ForceV a, ForceV b) { return ForceProd{a.v, b.v}; }
+__device__ __forceinline__ ForceProd operator*(float s, ForceV b) { return ForceProd{bc(s), b.v}; }
+__device__ __forceinline__ ForceV operator+(ForceV a, ForceV b) { return ForceV{a.v + b.v}; }
+__device__ __forceinline__ ForceV operator+(ForceV a, float s) { return ForceV{a.v + s}; }
+__device__ __forceinline__ ForceV operator+(ForceProd p, ForceV c) { return ForceV{fma2(p.a, p.b, c.v)}; }
+__device__ __forceinline__ ForceV operator+(ForceV c, ForceProd p) { return p + c; }
+__device__ __forceinline__ ForceV operator+(ForceProd p, ForceProd q) { return p + ForceV{q.a * q.b}; }
+__device__ __forceinline__ ForceV operator+(ForceProd p, float s) { return p + ForceV{bc(s)}; }
+__device__ __forceinline__ ForceV mms_rcp(ForceV a) { return ForceV{rcp2(a.v)}; }
+
+}  // namespace lbmv
+
+// the generated code needs mms_rcp
 #include "mms_force.cuh"
 
 namespace lbmv {
@@ -31,6 +62,7 @@ struct BatchLattice {
     int nx, ny, P;
     int tiles_x, strips, H;    // units: tiles_x x strips
     int unit0;                 // first unit of this lattice
+    const float2* trig;        // sin, cos of k y of the ny rows
     float s_e, s_eps, s_q, s_nu, h_e, h_eps, h_q, h_nu;
     float kappa, rho0;
     float k, w, A, U0, phi0, nu;   // manufactured solution
@@ -45,19 +77,6 @@ struct BatchParams {
     float scale, inv_scale;    // FP16 / BF16 deviation scale
     int* err;
 };
-
-// Eq. (25) force at a lane's two columns. Kept out of line: inlined into each of the
-// row loop's unrolled copies it makes the loop too large for the row states to stay
-// in registers.
-struct ForcePair {
-    V2 fx, fy;
-};
-__device__ __forceinline__ ForcePair mms_force_pair(V2 sx, V2 cx, float sy, float cy, float ct, float st, float k,
-                                                 float w, float A, float U0, float phi0, float nu) {
-    ForcePair r;
-    mms_force<V2>(sx, cx, bc(sy), bc(cy), ct, st, k, w, A, U0, phi0, nu, r.fx, r.fy);
-    return r;
-}
 
 // Per-unit view with the interface warp_run_strip expects.
 template <typename S>
@@ -89,6 +108,9 @@ struct BatchCtx {
     V2 sx2, cx2;               // sin, cos of k x of the lane's two columns
     float k, w, A, U0, phi0, nu, rho0;
     float ct, st, ct1;         // cos(wt), sin(wt), cos(w(t+1))
+    V2 asx, a1sx;              // A cos(wt) sin(kx), A cos(w(t+1)) sin(kx)
+    const float2* trig;        // sin, cos of k y of the rows (BatchLattice::trig)
+    mutable float2 next;       // those of the next row: on their way while a row is worked on
 
     __device__ __forceinline__ uint64_t* bar(int r) const { return reinterpret_cast<uint64_t*>(smem) + wslot(r); }
     __device__ __forceinline__ const S* pop(int r) const {
@@ -97,17 +119,30 @@ struct BatchCtx {
     __device__ __forceinline__ bool row_valid(int) const { return true; }
     static __device__ __forceinline__ constexpr int pop_stride() { return L::WW; }
 
-    __device__ __forceinline__ void row_setup(int r, PRow& st) const {
-        sincospif(2.0f * (float)r / (float)p.ny, &st.sy, &st.cy);
+    // the periodic image of row r (strips reach three rows beyond the lattice)
+    __device__ __forceinline__ int row(int r) const {
+        if (r < 0) { r += p.ny; if (r < 0) r = p.ny - 1 - ((-1 - r) % p.ny); }
+        else if (r >= p.ny) { r -= p.ny; if (r >= p.ny) r %= p.ny; }
+        return r;
     }
-    __device__ __forceinline__ V2 phi2(int, const PRow& st) const { return fma2(A * ct * st.sy, sx2, bc(phi0)); }
+    // rows come in order from y0 - 2 on (start_rows before the first): one load a row, used
+    // a row later, in the place of a sincospif in every lane (about 35 instructions)
+    __device__ __forceinline__ void start_rows() const { next = trig[row(y0 - 2)]; }
+    __device__ __forceinline__ void row_setup(int r, PRow& st) const {
+        st.sy = next.x;
+        st.cy = next.y;
+        next = trig[row(r + 1)];
+    }
+    __device__ __forceinline__ V2 phi2(int, const PRow& st) const { return fma2(st.sy, asx, bc(phi0)); }
     template <bool FAST>
-    __device__ __forceinline__ V2 phin2(int, const PRow& st) const { return fma2(A * ct1 * st.sy, sx2, bc(phi0)); }
+    __device__ __forceinline__ V2 phin2(int, const PRow& st) const { return fma2(st.sy, a1sx, bc(phi0)); }
     template <bool FAST>
     __device__ __forceinline__ void add_field_force(int, const PRow& st, V2& Fx, V2& Fy) const {
-        const ForcePair f = mms_force_pair(sx2, cx2, st.sy, st.cy, ct, this->st, k, w, A, U0, phi0, nu);
-        Fx = fma2(rho0, f.fx, Fx);
-        Fy = fma2(rho0, f.fy, Fy);
+        ForceV fx, fy;
+        mms_force<ForceV>(ForceV{sx2}, ForceV{cx2}, ForceV{bc(st.sy)}, ForceV{bc(st.cy)}, ct, this->st, k, w, A, U0,
+                          phi0, nu, fx, fy);
+        Fx = fma2(rho0, fx.v, Fx);
+        Fy = fma2(rho0, fy.v, Fy);
     }
 
     // this lane's part of staging a source row: lane 0 copies the nine population rows
@@ -129,9 +164,7 @@ struct BatchCtx {
     // all lanes: load source row r (periodic) into its slot
     __device__ __forceinline__ void issue(int r) {
         issued = r;
-        int gr = r % p.ny;
-        if (gr < 0) gr += p.ny;
-        cp.issue(lane, wslot(r), gr);
+        cp.issue(lane, wslot(r), row(r));
     }
     __device__ __forceinline__ void wait_upto(int r) {
         r = min(r, rhi);
@@ -177,6 +210,8 @@ __global__ void __launch_bounds__(32, MINB) vanse_batch_kernel(const __grid_cons
         fence_mbar_init();
     }
     __syncwarp();
+    pdl_wait();
+    pdl_next();
     const int t = *bp.clock;
     uint32_t phase = 0;
     for (;;) {
@@ -247,6 +282,10 @@ __global__ void __launch_bounds__(32, MINB) vanse_batch_kernel(const __grid_cons
         sincospif(2.0f * (float)(c.xa + 1) / (float)Lt.nx, &sb_, &cb_);
         c.sx2 = mk(sa_, sb_);
         c.cx2 = mk(ca_, cb_);
+        c.asx = (Lt.A * c.ct) * c.sx2;
+        c.a1sx = (Lt.A * c.ct1) * c.sx2;
+        c.trig = Lt.trig;
+        c.start_rows();
         c.rlo = c.y0 - 3;
         c.rhi = c.y1 + 2;
         c.waited = c.rlo - 1;
@@ -269,21 +308,34 @@ __global__ void __launch_bounds__(32, MINB) vanse_batch_kernel(const __grid_cons
     }
 }
 
-// After each batched step, before the tick: refresh the periodic ghost columns of the
-// buffer every lattice's step just wrote (blockIdx.y = lattice).
+// After each batched step: refresh the periodic ghost columns of the buffer every lattice's
+// step just wrote (blockIdx.y = lattice); the CTA that finishes last advances the clock
+// (clock[0]) and re-arms the unit counter (clock[1]) and its own count of CTAs (clock[3]).
+// 32-bit indices: 54 n values, n at most 65536.
 template <typename S>
-__global__ void batch_ghost_fill_kernel(const BatchLattice* lats, const int* clock) {
+__global__ void batch_ghost_fill_kernel(const BatchLattice* lats, int* clock) {
+    pdl_wait();
+    pdl_next();
     const BatchLattice& L = lats[blockIdx.y];
     S* buf = reinterpret_cast<S*>(L.buf[(*clock + 1) & 1]);
-    const long long n = 9LL * L.ny * 2 * kGhost;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
+    const unsigned n = 54u * (unsigned)L.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
         fill_ghosts<S>(buf, L.plane, L.nx, L.ny, L.P, k);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(clock + 3, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+            clock[0] += 1;
+            clock[1] = 0;
+            clock[3] = 0;
+        }
+    }
 }
 
-// After each batched step: advance the clock and re-arm the unit counter.
-__global__ void batch_tick_kernel(int* clock, int* counter) {
-    *clock += 1;
-    *counter = 0;
+// sin, cos of k y of a lattice's rows (BatchLattice::trig), as the read-back evaluates them
+__global__ void batch_trig_kernel(float2* trig, int n) {
+    for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x)
+        sincospif(2.0f * (float)y / (float)n, &trig[y].x, &trig[y].y);
 }
 
 }  // namespace lbmv
@@ -544,6 +596,10 @@ __global__ void __launch_bounds__(32, MINB) vanse_batch_one_kernel(const __grid_
     sincospif(2.0f * (float)(c.xa + 1) / (float)Lt.nx, &sb_, &cb_);
     c.sx2 = mk(sa_, sb_);
     c.cx2 = mk(ca_, cb_);
+    c.asx = (Lt.A * c.ct) * c.sx2;
+    c.a1sx = (Lt.A * c.ct1) * c.sx2;
+    c.trig = Lt.trig;
+    c.start_rows();
     c.rlo = c.y0 - 3;
     c.rhi = c.y1 + 2;
     c.waited = c.rlo - 1;
