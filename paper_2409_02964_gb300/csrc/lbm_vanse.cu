@@ -260,7 +260,10 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
 // 185.9 / 165.8 / 164.4 / 164.2 (five waves of at least 16 rows, the rule before: 21.5,
 // 36.1, 48.1, 72.9, 110.2, 170.1). With solid cells kernel 5 cuts ten waves of at least 16
 // rows: the CTAs next to a solid take several times as long as the others, and shorter
-// strips shorten the longest CTA. FP64 on kernel 1: march64_us. Otherwise (kernels 1 to 4):
+// strips shorten the longest CTA. FP64 on kernel 1: march64_us; with solid cells only where
+// 16-row strips are fewer than two per SM and no kernel was asked for (us a step, generic
+// strips / march64_us: 39 x 17 262 / 50, 150 x 90 421 / 78, 400 x 300 390 / 205, 838 x 226
+// 377 / 266, but 900 x 900 732 / 801). Otherwise (kernels 1 to 4):
 // five waves of at least 16 rows.
 //
 // march64_us: a CTA (128 threads) keeps an SM's FP64 pipe 5/6 busy by itself, 7.8 us a row,
@@ -284,7 +287,8 @@ void pick_strip_height(lbm_vanse* h) {
         int w = 1;
         while (w < 5 && rows(w) > kWaveRows[w - 1]) ++w;
         H = rows(w);
-    } else if (H <= 0 && h->prm.storage == LBM_FP64 && !h->has_solid) {
+    } else if (H <= 0 && h->prm.storage == LBM_FP64 &&
+               (!h->has_solid || (h->auto_kernel && (long long)h->gridx * ((h->prm.ny + 15) / 16) < 2LL * h->nsm))) {
         H = 1;
         for (int k = 2; k <= std::min(h->prm.ny, 128); ++k)
             if (march64_us(h, k) < march64_us(h, H)) H = k;
