@@ -137,6 +137,9 @@ lbm_status lbm_vanse_set_void_fraction_f32(lbm_vanse_t h, const float* phi_t, co
  * next call. */
 lbm_status lbm_vanse_set_body_force(lbm_vanse_t h, double gx, double gy, const double* field,
                                     int on_device);
+/* The same with a float field: padded as it is (FP64 storage widens it exactly). */
+lbm_status lbm_vanse_set_body_force_f32(lbm_vanse_t h, double gx, double gy, const float* field,
+                                        int on_device);
 
 /* Linear drag added to the body force (Sec. 3.1, Eq. 21 and 23):
  *   F^B += -beta (u - u_s),  beta(x) = phi(x)^2 (d0 + d1 (1 - phi(x))),

@@ -23,7 +23,7 @@ STATUS_NAMES = {0: "LBM_OK", -1: "LBM_ERR_ARG", -2: "LBM_ERR_CUDA", -3: "LBM_ERR
 EXPORTS = [
     "lbm_vanse_default_params", "lbm_vanse_create", "lbm_vanse_set_void_fraction",
     "lbm_vanse_set_void_fraction_f32", "lbm_vanse_reduce_async", "lbm_vanse_step_sums",
-    "lbm_vanse_set_body_force", "lbm_vanse_set_drag", "lbm_vanse_set_moving_wall", "lbm_vanse_set_solid_cells",
+    "lbm_vanse_set_body_force", "lbm_vanse_set_body_force_f32", "lbm_vanse_set_drag", "lbm_vanse_set_moving_wall", "lbm_vanse_set_solid_cells",
     "lbm_vanse_set_row_wait_limit", "lbm_vanse_state_bytes", "lbm_vanse_save_state", "lbm_vanse_load_state",
     "lbm_vanse_init_fields",
     "lbm_vanse_step", "lbm_vanse_macros",
@@ -126,6 +126,7 @@ def load(path: str | None = None):
         "lbm_vanse_reduce_async": (i, [vp, vp, i]),
         "lbm_vanse_step_sums": (i, [vp, vp, i]),
         "lbm_vanse_set_body_force": (i, [vp, d, d, vp, i]),
+        "lbm_vanse_set_body_force_f32": (i, [vp, d, d, vp, i]),
         "lbm_vanse_set_drag": (i, [vp, d, d, d, d]),
         "lbm_vanse_set_moving_wall": (i, [vp, i, d, d]),
         "lbm_vanse_set_solid_cells": (i, [vp, i]),

@@ -30,6 +30,9 @@ def _check(st: int, handle) -> None:
         raise LbmError(st, msg.decode() if msg else "")
 
 
+_TORCH = {np.float64: torch.float64, np.float32: torch.float32}
+
+
 class _Arg:
     """Holds a caller array as (pointer, on_device) for one call, converted to
     ``dtype`` (float64, or float32 for the entry points that take floats)."""
@@ -41,7 +44,9 @@ class _Arg:
         if isinstance(a, torch.Tensor) and a.is_cuda:
             if a.device != device:
                 raise ValueError(f"tensor on {a.device}, lattice on {device}")
-            t = a.detach().to({np.float64: torch.float64, np.float32: torch.float32}[dtype]).contiguous()
+            t = a
+            if a.dtype is not _TORCH[dtype] or not a.is_contiguous():
+                t = a.detach().to(_TORCH[dtype]).contiguous()
             if t.numel() != count:
                 raise ValueError(f"expected {count} elements, got {t.numel()}")
             self.ptr, self.on_device, self._keep = t.data_ptr(), 1, t
@@ -149,8 +154,11 @@ class Lattice:
         _check(fn(self._h, a.ptr, b.ptr, a.on_device), self._h)
 
     def set_body_force(self, gx: float = 0.0, gy: float = 0.0, field=None) -> None:
-        a = _Arg(field, 2 * self.n, self.device)
-        _check(self._L.lbm_vanse_set_body_force(self._h, float(gx), float(gy), a.ptr, a.on_device), self._h)
+        """A float32 field (numpy or torch) goes through lbm_vanse_set_body_force_f32."""
+        f32 = _is_f32(field)
+        a = _Arg(field, 2 * self.n, self.device, np.float32 if f32 else np.float64)
+        fn = self._L.lbm_vanse_set_body_force_f32 if f32 else self._L.lbm_vanse_set_body_force
+        _check(fn(self._h, float(gx), float(gy), a.ptr, a.on_device), self._h)
 
     def set_drag(self, d0: float = 0.0, d1: float = 0.0, us_x: float = 0.0, us_y: float = 0.0) -> None:
         """F^B += -beta (u - u_s), beta = phi^2 (d0 + d1 (1 - phi)) (lbm_vanse_set_drag)."""
