@@ -19,8 +19,8 @@
 // Bound by issue and latency (two warps per scheduler, the force on top of the collision).
 // us per step, before / after the force in 53 packed operations instead of 170, tabulated
 // row sines, unit heights by schedule and one launch fewer (before: units of 48 rows): 24
-// lattices of 10.96 M cells FP32 205 / 188, FP16 214 / 179, 40 of 12.6 M FP32 260 / 202,
-// 40 of 17.0 M BF16 327 / 267, 7 of 2.3 M FP32 68.6 / 52.9.
+// lattices of 10.96 M cells FP32 205 / 184, FP16 214 / 171, 40 of 12.6 M FP32 260 / 197,
+// 40 of 17.0 M BF16 327 / 262, 7 of 2.3 M FP32 68.6 / 45.8.
 #pragma once
 
 #include "vanse_aux.cuh"
