@@ -74,8 +74,13 @@ __global__ void ghost_fill_kernel(S* __restrict__ buf, long long plane, int nx, 
     pdl_wait();
     pdl_next();
     const long long n = (long long)npl * ny * 2 * kGhost;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-        fill_ghosts<S>(buf, plane, nx, ny, P, k);
+    if (n < (1LL << 31)) {   // (32-bit divisions)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < (unsigned)n; k += gridDim.x * blockDim.x)
+            fill_ghosts<S>(buf, plane, nx, ny, P, k);
+    } else {
+        for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
+            fill_ghosts<S>(buf, plane, nx, ny, P, k);
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) *step_next = *step_ctr + 1u;
 }
 
