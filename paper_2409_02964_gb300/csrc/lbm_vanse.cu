@@ -13,8 +13,8 @@
 #include <cstring>
 #include <mutex>
 #include <functional>
+#include <map>
 #include <numeric>
-#include <queue>
 #include <string>
 #include <vector>
 #include <type_traits>
@@ -1682,7 +1682,6 @@ struct lbm_vanse_batch {
     BatchLattice* d_desc = nullptr;
     int* d_units = nullptr;              // lattice of each unit
     int* d_clock = nullptr;              // [0] = t, [1] = unit counter, [2] = error flag, [3] = ghost CTAs done
-    float2* d_trig = nullptr;            // BatchLattice::trig of every lattice
     double* scratch = nullptr;           // dense rho of the largest lattice
     double* partial = nullptr;
     double* red_out = nullptr;
@@ -1760,14 +1759,18 @@ int batch_rows(const lbm_vanse_batch* b) {
             cost = sum / b->grid + H + 6;
         } else {
             std::sort(kinds.begin(), kinds.end(), std::greater<>());
-            std::priority_queue<int, std::vector<int>, std::greater<int>> free_at;
+            // CTAs by the time they fall free (whole groups of them take units of one height)
+            std::map<int, long long> free_at{{0, b->grid}};
             int end = 0;
             for (auto& k : kinds)
-                for (long long u = 0; u < k.second; ++u) {
-                    int at = 0;
-                    if ((int)free_at.size() >= b->grid) { at = free_at.top(); free_at.pop(); }
-                    free_at.push(at + k.first);
-                    end = std::max(end, at + k.first);
+                for (long long left = k.second; left > 0;) {
+                    const auto first = free_at.begin();
+                    const long long m = std::min(left, first->second);
+                    const int t = first->first + k.first;
+                    if ((first->second -= m) == 0) free_at.erase(first);
+                    free_at[t] += m;
+                    end = std::max(end, t);
+                    left -= m;
                 }
             cost = end;
         }
@@ -2030,14 +2033,10 @@ extern "C" lbm_status lbm_vanse_batch_create(const lbm_vanse_batch_lattice* latt
         }
         long long rows = 0;
         for (auto& q : b->lat) rows += q.n;
-        e = cudaMalloc((void**)&b->d_desc, count * sizeof(BatchLattice));
-        if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_trig, rows * sizeof(float2));
-        float2* tr = b->d_trig;
-        for (int i = 0; i < count && e == cudaSuccess; tr += b->lat[i].n, ++i) {
-            b->desc[i].trig = tr;
-            batch_trig_kernel<<<(b->lat[i].n + 127) / 128, 128, 0, b->stream>>>(tr, b->lat[i].n);
-            e = cudaGetLastError();
-        }
+        // the descriptors, and behind them the row sines of every lattice
+        e = cudaMalloc((void**)&b->d_desc, count * sizeof(BatchLattice) + rows * sizeof(float2));
+        float2* tr = (float2*)(b->d_desc + count);
+        for (int i = 0; i < count; tr += b->lat[i].n, ++i) b->desc[i].trig = tr;
         if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_clock, 4 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_clock, 0, 4 * sizeof(int), b->stream);
         if (e == cudaSuccess) e = cudaMalloc((void**)&b->scratch, (size_t)nmax * nmax * sizeof(double));
@@ -2047,6 +2046,11 @@ extern "C" lbm_status lbm_vanse_batch_create(const lbm_vanse_batch_lattice* latt
     }
     if (st == LBM_OK) st = BDISPATCH(b, batch_configure);
     if (st == LBM_OK) st = batch_decompose(b, p->strip_rows > 0 ? p->strip_rows : batch_rows(b));
+    if (st == LBM_OK) {
+        batch_trig_kernel<<<count, 256, 0, b->stream>>>(b->d_desc);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) st = bfail(nullptr, LBM_ERR_CUDA, "batch sines: %s", cudaGetErrorString(e));
+    }
     if (st != LBM_OK) {
         if (b->msg.size()) g_create_error = b->msg;
         lbm_vanse_batch_destroy(b);
@@ -2147,7 +2151,7 @@ extern "C" void lbm_vanse_batch_destroy(lbm_vanse_batch_t b) {
     cudaStreamSynchronize(b->stream);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    void* ptrs[] = {b->pool, b->d_desc, b->d_units, b->d_clock, b->d_trig, b->scratch, b->partial, b->red_out};
+    void* ptrs[] = {b->pool, b->d_desc, b->d_units, b->d_clock, b->scratch, b->partial, b->red_out};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete b;

@@ -332,10 +332,13 @@ __global__ void batch_ghost_fill_kernel(const BatchLattice* lats, int* clock) {
     }
 }
 
-// sin, cos of k y of a lattice's rows (BatchLattice::trig), as the read-back evaluates them
-__global__ void batch_trig_kernel(float2* trig, int n) {
-    for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x)
-        sincospif(2.0f * (float)y / (float)n, &trig[y].x, &trig[y].y);
+// sin, cos of k y of every lattice's rows (BatchLattice::trig; blockIdx.x = lattice), as the
+// read-back evaluates them
+__global__ void batch_trig_kernel(const BatchLattice* lats) {
+    const BatchLattice& L = lats[blockIdx.x];
+    float2* trig = const_cast<float2*>(L.trig);
+    for (int y = threadIdx.x; y < L.ny; y += blockDim.x)
+        sincospif(2.0f * (float)y / (float)L.ny, &trig[y].x, &trig[y].y);
 }
 
 }  // namespace lbmv
