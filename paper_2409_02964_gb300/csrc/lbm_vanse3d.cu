@@ -656,8 +656,10 @@ __global__ void v3_rebase(const double* __restrict__ phin_src, T* __restrict__ p
 
 template <typename Tin, typename Tout>
 __global__ void v3_convert(const Tin* __restrict__ a, Tout* __restrict__ b, long long n, double offset = 0.0) {
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-        b[k] = (Tout)((double)a[k] + offset);
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+        const double v = widen(a[k]);
+        b[k] = (Tout)(offset == 0.0 ? v : v + offset);
+    }
 }
 
 // FP64 mass and momentum sums: out[0..3] += per-block partials
