@@ -1,9 +1,10 @@
 """Compile the CUDA library ``liblbm_vanse.so`` for sm_103a, in-tree.
 
-Two translation units, compiled in parallel and linked into one shared library in
-``paper_2409_02964_gb300/_build/`` with nvcc for ``arch=compute_103a,code=sm_103a``:
-``csrc/lbm_vanse.cu`` (the C ABI of ``include/lbm_vanse.h`` and the D2Q9 kernels) and
-``csrc/lbm_vanse3d.cu`` (``include/lbm_vanse3d.h``, the D3Q19 step).
+The translation units of ``csrc/`` are compiled in parallel and linked into one shared
+library in ``paper_2409_02964_gb300/_build/`` with nvcc for ``arch=compute_103a,
+code=sm_103a``: ``lbm_vanse.cu`` (the C ABI of ``include/lbm_vanse.h`` and most D2Q9
+kernels), ``vanse_warp_*.cu`` and ``vanse_tile.cu`` (instances of the one-warp and the tile
+kernels) and ``lbm_vanse3d.cu`` (``include/lbm_vanse3d.h``, the D3Q19 step).
 """
 from __future__ import annotations
 
