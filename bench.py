@@ -348,7 +348,7 @@ def batch_run(steps: int = 2000, count: int = 512, each_steps: int = 200):
                      "solves_per_s": round(count * ns / steps / secs, 2),
                      "MLUPS": round(b.cells * ns / secs / 1e6, 1),
                      "GB_s": round(72 * b.cells * ns / secs / 1e9, 1),
-                     "gpu_launches": ns * (3 if mode == "persistent" else count + 2)}
+                     "gpu_launches": ns * (2 if mode == "persistent" else count + 1)}
         if mode == "persistent":
             errs = np.array([b.relative_error(i) for i in range(count)])
     out = {"workload": BATCH_WORKLOAD, "lattices": count, "cells": b.cells, "steps": steps,
@@ -422,10 +422,10 @@ def adjoint_run(n: int = 1024, nsteps: int = 4000, avg: int = 100, ckpt: int = 2
         ch = P.Channel(nx=n, ny=n, nsteps=nsteps, avg_steps=avg, checkpoint_every=ckpt, dense_segments=dense)
         J, g, st = P.outlet_momentum(phi, ch)
         fwd_s, bwd_s = st["forward_ms"] / 1e3, st["backward_ms"] / 1e3
-        # FP64 flops per cell: a forward step 598; a backward step with its segment
-        # recompute 1614 (ncu instruction counts of the adjoint kernels); the two-level
-        # scheme recomputes every step once more (598)
-        flops = 598.0 + 1614.0 + (0.0 if dense else 598.0)
+        # FP64 flops per cell: a forward step 263; a backward step with its segment
+        # recompute 632 (ncu instruction counts of the adjoint kernels); the two-level
+        # scheme recomputes every step once more (263)
+        flops = 263.0 + 632.0 + (0.0 if dense else 263.0)
         achieved = flops * lups / (fwd_s + bwd_s) / 1e12
         out[name] = {"J": J, "max_abs_grad": float(g.abs().max()),
                      "forward_s": round(fwd_s, 3), "backward_s": round(bwd_s, 3),
