@@ -303,7 +303,12 @@ void pick_strip_height(lbm_vanse* h) {
 
 // The tile kernel (vanse_tile.cuh) instead of kernel 5, for lattices that did not ask for
 // a kernel or a strip height: small ones, where a strip's serial rows are the step's time,
-// and every one with solid cells, whose marching strips are as slow as their slowest row.
+// and those with solid cells up to 4.5 M cells (FP16 / BF16 4 M), whose marching strips are as
+// slow as their slowest row. Beyond, a lattice whose solid cells lie together marches most of
+// its strips on the solid-free path, quicker than tiles (us a step, tiles / marching, one
+// block of solid cells: 1531 x 1024 FP32 44.9 / 93.8, 2048^2 110 / 129, 2500^2 157 / 148,
+// 4096^2 406 / 302, FP16 1600^2 84 / 103, 2048^2 135 / 131; with scattered ones as well 2500^2
+// FP32 188 / 228, 4096^2 488 / 590: the host does not know which it has).
 // Rows per CTA and instance: R = 4 without spills while all CTAs fit at once (two per
 // SM), R = 4 of the 80-register instance while three per SM hold them, else R = 8. Without
 // solid cells up to two waves of the last (512^2 9.7 us against 11.1 for the marching
@@ -313,6 +318,7 @@ void pick_tile(lbm_vanse* h) {
     auto ctas = [&](int R) { return (long long)h->gridx * ((h->prm.ny + R - 1) / R); };
     h->tile_rows = 0;
     if (!h->has_solid && ctas(8) > 4LL * nsm) return;
+    if (h->has_solid && (double)h->prm.nx * h->prm.ny > (h->sbytes == 4 ? 4.5e6 : 4.0e6)) return;
     h->tile_big = ctas(4) > 2LL * nsm;
     h->tile_rows = ctas(4) <= 3LL * nsm ? 4 : 8;
 }

@@ -36,3 +36,24 @@ def test_short_strips_equal_tall_ones(nx, ny, wall):
         lat.sync()
         lat.close()
     assert bool(torch.isfinite(got[0]).all()) and torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("storage,nx,ny,tiles", [("fp32", 2250, 2000, True), ("fp32", 2251, 2000, False),
+                                                 ("fp16", 2000, 2000, True), ("fp16", 2001, 2000, False)])
+def test_large_lattices_with_solids_march(storage, nx, ny, tiles):
+    """On both sides of the line between tiles and the marching kernel: which of them runs
+    (only the marching kernel waits for staged rows, so only it can time out)."""
+    import paper_2409_02964_gb300 as P
+    phi = np.full((ny, nx), 0.7)
+    phi[40:60, 100:130] = 0.0
+    zero = np.zeros((ny, nx))
+    lat = P.Lattice(nx, ny, 0.7, storage=storage)
+    lat.set_solid_cells()
+    lat.set_void_fraction(phi)
+    lat.init_fields(np.ones((ny, nx)), zero, zero)
+    lat.step(1)
+    lat.sync()
+    lat._L.lbm_vanse_set_row_wait_limit(lat._h, 0)
+    lat.step(1)
+    assert (lat._L.lbm_vanse_sync(lat._h) == -6) is not tiles     # LBM_ERR_TIMEOUT
+    lat.close()
