@@ -21,6 +21,7 @@
 #include <utility>
 
 #include "lbm_vanse.h"
+#include "step_rules.h"
 #include "vanse_adjoint.cuh"
 #include "vanse_aux.cuh"
 #include "vanse_batch.cuh"
@@ -250,94 +251,21 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
     return (const void*)vanse_step_kernel<S, R, kThreads>;
 }
 
-// Rows per strip (CTA): strip_rows, or automatic. A strip of H rows steps through H + 6
-// (kernel 5: 0.9 us a row with one warp or eight per SM), so few waves of tall strips cost
-// fewer halo rows, while several waves of short ones keep the memory busier and end more
-// evenly. Kernel 5 takes the fewest waves w whose strips stay within kWaveRows[w]; FP32
-// step on one GB300 in us, strips of 1 / 2 / 3 / 5 waves: 800^2 16.2 / 19.8 / 22.8 / -,
-// 1531 x 1024 30.0 / 30.4 / 36.1 / 40, 1800 x 1400 42.4 / 42.1 / 46.3 / 53.7, 2048^2
-// 72.2 / 64.9 / 66.4 / 72.6, 3000 x 2500 119 / 105.7 / 104.2 / 110.1, 4001 x 3001
-// 185.9 / 165.8 / 164.4 / 164.2 (five waves of at least 16 rows, the rule before: 21.5,
-// 36.1, 48.1, 72.9, 110.2, 170.1). With solid cells kernel 5 cuts ten waves of at least 16
-// rows: the CTAs next to a solid take several times as long as the others, and shorter
-// strips shorten the longest CTA. FP64 on kernel 1: march64_us; with solid cells only where
-// 16-row strips are fewer than two per SM and no kernel was asked for (us a step, generic
-// strips / march64_us: 39 x 17 262 / 50, 150 x 90 421 / 78, 400 x 300 390 / 205, 838 x 226
-// 377 / 266, but 900 x 900 732 / 801). Otherwise (kernels 1 to 4):
-// five waves of at least 16 rows.
-//
-// march64_us: a CTA (128 threads) keeps an SM's FP64 pipe 5/6 busy by itself, 7.8 us a row,
-// and two on an SM take 13 us a row; a strip of H rows steps through about H + 4. FP64
-// step in us, H = 12 / 16 / 24 / 48: 1024 x 768 380 / 472 / 365 / 406, 2000 x 1500 1317 /
-// 1400 / 1383 / 1392.
-double march64_us(const lbm_vanse* h, int H) {
-    const long long ctas = (long long)h->gridx * ((h->prm.ny + H - 1) / H), slots = 2LL * h->nsm;
-    const long long rem = ctas % slots;
-    return (H + 4) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= h->nsm ? 7.8 : 13.0)));
+// The launch rules of step_rules.h on this handle.
+StepShape step_shape(const lbm_vanse* h) {
+    return StepShape{h->prm.nx, h->prm.ny, h->gridx,      h->resident,  h->nsm,
+                     h->kernel, h->sbytes, h->prm.strip_rows, h->has_solid, h->auto_kernel};
 }
 
 void pick_strip_height(lbm_vanse* h) {
-    static const int kWaveRows[4] = {24, 36, 40, 44};
-    int H = h->prm.strip_rows;
-    auto rows = [&](int waves) {
-        const int nstrips = std::max(1, waves * h->resident / h->gridx);
-        return (h->prm.ny + nstrips - 1) / nstrips;
-    };
-    if (H <= 0 && h->kernel == 5 && !h->has_solid) {
-        int w = 1;
-        while (w < 5 && rows(w) > kWaveRows[w - 1]) ++w;
-        H = rows(w);
-    } else if (H <= 0 && h->prm.storage == LBM_FP64 &&
-               (!h->has_solid || (h->auto_kernel && (long long)h->gridx * ((h->prm.ny + 15) / 16) < 2LL * h->nsm))) {
-        H = 1;
-        for (int k = 2; k <= std::min(h->prm.ny, 128); ++k)
-            if (march64_us(h, k) < march64_us(h, H)) H = k;
-    } else if (H <= 0) {
-        const int waves = (h->has_solid && h->kernel == 5) ? 10 : 5;
-        const int nstrips = std::max(1, (waves * h->resident + h->gridx - 1) / h->gridx);
-        H = std::max((h->prm.ny + nstrips - 1) / nstrips, 16);
-    }
-    h->H = std::min(H, h->prm.ny);
+    h->H = strip_height(step_shape(h));
     h->gridy = (h->prm.ny + h->H - 1) / h->H;
 }
 
-// The tile kernel (vanse_tile.cuh) instead of kernel 5, for lattices that did not ask for
-// a kernel or a strip height: small ones, where a strip's serial rows are the step's time,
-// and those with solid cells up to 4.5 M cells (FP16 / BF16 4 M), whose marching strips are as
-// slow as their slowest row. Beyond, a lattice whose solid cells lie together marches most of
-// its strips on the solid-free path, quicker than tiles (us a step, tiles / marching, one
-// block of solid cells: 1531 x 1024 FP32 44.9 / 93.8, 2048^2 110 / 129, 2500^2 157 / 148,
-// 4096^2 406 / 302, FP16 1600^2 84 / 103, 2048^2 135 / 131; with scattered ones as well 2500^2
-// FP32 188 / 228, 4096^2 488 / 590: the host does not know which it has).
-// Rows per CTA and instance: R = 4 without spills while all CTAs fit at once (two per
-// SM), R = 4 of the 80-register instance while three per SM hold them, else R = 8. Without
-// solid cells up to two waves of the last (512^2 9.7 us against 11.1 for the marching
-// kernel in strips of 4 rows, 640^2 12.8 against 11.9).
 void pick_tile(lbm_vanse* h) {
-    const int nsm = h->nsm;
-    auto ctas = [&](int R) { return (long long)h->gridx * ((h->prm.ny + R - 1) / R); };
-    h->tile_rows = 0;
-    if (!h->has_solid && ctas(8) > 4LL * nsm) return;
-    if (h->has_solid && (double)h->prm.nx * h->prm.ny > (h->sbytes == 4 ? 4.5e6 : 4.0e6)) return;
-    h->tile_big = ctas(4) > 2LL * nsm;
-    h->tile_rows = ctas(4) <= 3LL * nsm ? 4 : 8;
-}
-
-// The FP64 tile kernel instead of kernel 1 where it is quicker: rows per CTA by the FP64
-// pipe time of the busiest SM, CTAs per SM times kUs[R] (measured on 2000 x 1500; the same
-// figure predicts every size within 10 %). FP64 step in us, tiles / kernel 1 at 16 rows:
-// 64^2 9.6 / 137 (R = 2), 130 x 71 10 / 144 (R = 3), 256^2 40 / 145 (R = 6), 512^2 133 /
-// 246 (R = 8); 1024 x 768 398 / 365 at 24 rows.
-void pick_tile64(lbm_vanse* h) {
-    static const struct { int rows; double us; } kUs[] = {{1, 4.0}, {2, 5.8}, {3, 7.2}, {4, 8.7}, {6, 13.2}, {8, 16.6}};
-    const long long tx = (h->prm.nx + kTile64Cols - 1) / kTile64Cols;
-    double best = march64_us(h, h->H);
-    h->tile_rows = 0;
-    for (const auto& k : kUs) {
-        const long long ctas = tx * ((h->prm.ny + k.rows - 1) / k.rows);
-        const double us = k.us * (double)((ctas + h->nsm - 1) / h->nsm);
-        if (us < best) { best = us; h->tile_rows = k.rows; }
-    }
+    const TileShape t = tile_shape(step_shape(h));
+    h->tile_rows = t.rows;
+    h->tile_big = t.big;
 }
 
 template <typename S>
@@ -365,7 +293,7 @@ lbm_status configure(lbm_vanse* h) {
             pick_tile(h);
         }
     } else if (h->auto_kernel && h->prm.bc_x != LBM_BC_BOUNCEBACK && h->prm.eq_order != 2 && h->prm.strip_rows == 0) {
-        pick_tile64(h);
+        h->tile_rows = tile64_rows(step_shape(h), h->H);
     }
     return LBM_OK;
 }

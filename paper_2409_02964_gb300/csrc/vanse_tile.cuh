@@ -17,6 +17,7 @@
 // advances the step counter of the stochastic rounding, so a step is one launch.
 #pragma once
 
+#include "step_rules.h"
 #include "vanse_warp.cuh"
 
 namespace lbmv {
@@ -223,7 +224,7 @@ struct TileCtx64 {
     }
 };
 
-constexpr int kTile64Cols = 28, kTile64Rows = 8;
+constexpr int kTile64Rows = 8;   // kTile64Cols: step_rules.h
 constexpr size_t tile64_smem_bytes(int warps) { return (size_t)10 * warps * 32 * sizeof(double); }
 
 cudaError_t tile64_launch(const StepParams<double>& p, cudaStream_t stream);
