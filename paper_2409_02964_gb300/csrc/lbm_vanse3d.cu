@@ -32,7 +32,7 @@
 
 namespace lbmv3 {
 
-using lbmv::rcp_nr;
+using lbmv::Divisor;
 using lbmv::widen;
 
 constexpr int Q = 19;
@@ -202,7 +202,7 @@ __global__ void v3_moments(const T* __restrict__ f, const T* __restrict__ phi, T
             d9 = v[17] - v[18];
     const T jx = (v[1] - v[2]) + ((d4 + d5) + (d6 + d7)), jy = (v[3] - v[4]) + ((d4 - d5) + (d8 + d9)),
             jz = (v[5] - v[6]) + ((d6 - d7) + (d8 - d9));
-    rho[c] = m0 * rcp_nr(phi[c]);
+    rho[c] = Divisor<T>(phi[c])(m0);
     j[c] = jx;
     j[g.N + c] = jy;
     j[2 * g.N + c] = jz;
@@ -261,14 +261,15 @@ __global__ void __launch_bounds__(128)
         const T drho = rc;      // rho - rho0 of plane p - 1
         rc = r;
         if (!out) continue;
-        const T im0 = rcp_nr(ph * (rho0 + drho)), k36 = (kappa - ph) * ((T)1 / (T)36);
+        const Divisor<T> by_m0(ph * (rho0 + drho));
+        const T k36 = (kappa - ph) * ((T)1 / (T)36);
         const T Gb[3] = {gx, gy, gz};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             T Fa = k36 * G[a] + ph * Gb[a];
             if (fb) Fa += fc[a];
             F[a * g.N + c] = Fa;
-            u[a * g.N + c] = (jc[a] + (T)0.5 * Fa) * im0;
+            u[a * g.N + c] = by_m0(jc[a] + (T)0.5 * Fa);
         }
     }
 }
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(TX * TY, 2)
 
         // C (x 12 undone here)
         const T tw = (T)1 / (T)12;
-        const T r = R.rho0 + dr, iph = rcp_nr(ph), X = kappa * iph, kr = (kappa - ph) * r;
+        const T r = R.rho0 + dr, X = Divisor<T>(ph)(kappa), kr = (kappa - ph) * r;
         const T kr23 = (T)2 / (T)3 * kr;
         const T C1 = (T)19 * (tw * (((T)1 - X) * G[9] + kr23 * ((G[0] + G[1]) + G[2])) - X * r * dtphi);
         const T dgx = tw * (G[6] + kr23 * G[0]), dgy = tw * (G[7] + kr23 * G[1]), dgz = tw * (G[8] + kr23 * G[2]);

@@ -436,7 +436,7 @@ __global__ void rho_kernel(const S* __restrict__ buf, const R* __restrict__ phi,
 #pragma unroll
             for (int i = 0; i < 9; ++i) s += f[i];
         }
-        rho[k] = (L.has_solid && ph == 0.0) ? 0.0 : s * rcp_nr(ph);
+        rho[k] = (L.has_solid && ph == 0.0) ? 0.0 : Divisor<double>(ph)(s);
     }
 }
 
@@ -471,9 +471,9 @@ __global__ void vel_kernel(const S* __restrict__ buf, const R* __restrict__ phi,
                 Fy = fma(beta, L.us_y, Fy);
                 m0 = fma(0.5, beta, m0);
             }
-            const double inv = rcp_nr(m0);
-            if (ux) ux[k] = fma(0.5, Fx, jx) * inv;
-            if (uy) uy[k] = fma(0.5, Fy, jy) * inv;
+            const Divisor<double> by_m0(m0);
+            if (ux) ux[k] = by_m0(fma(0.5, Fx, jx));
+            if (uy) uy[k] = by_m0(fma(0.5, Fy, jy));
             if (pr) pr[k] = r * (1.0 / 3.0);
             continue;
         }

@@ -36,19 +36,39 @@ template <> struct Prec<__nv_bfloat16> { using R = float; static constexpr bool 
 
 template <typename R> __device__ __forceinline__ R to_r(double v) { return (R)v; }
 
-// 1 / a by Newton-Raphson from the approximate reciprocal instruction: two steps in FP64
-// (4 FP64 operations; a correctly rounded division takes about ten, and the FP64 pipe, 2
-// lanes a cycle and SM, is what bounds the FP64 kernels), one in FP32.
-__device__ __forceinline__ double rcp_nr(double a) {
+// Division by a through Newton-Raphson from the approximate reciprocal instruction: two steps
+// in FP64 (4 FP64 operations; a correctly rounded division takes about ten, and the FP64 pipe,
+// 2 lanes a cycle and SM, is what bounds the FP64 kernels), one in FP32. The instruction
+// flushes subnormals, and the steps turn its zeros and infinities into NaN, so a divisor that
+// is zero, subnormal, infinite, NaN or has a subnormal reciprocal (told by its exponent bits
+// alone) takes the division instead.
+__device__ __forceinline__ double rcp_steps(double a) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
     r = fma(r, fma(-a, r, 1.0), r);
     return fma(r, fma(-a, r, 1.0), r);
 }
-__device__ __forceinline__ float rcp_nr(float a) {
+__device__ __forceinline__ float rcp_steps(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return fmaf(r, fmaf(-a, r, 1.0f), r);
+}
+// whether a and 1 / a are normal: biased exponent 1 .. 2044 (1 .. 252)
+__device__ __forceinline__ bool rcp_normal(double a) {
+    return (((uint32_t)__double2hiint(a) >> 20) & 0x7ffu) - 1u < 2044u;
+}
+__device__ __forceinline__ bool rcp_normal(float a) { return ((__float_as_uint(a) >> 23) & 0xffu) - 1u < 252u; }
+
+template <typename T>
+struct Divisor {
+    T a, r;
+    bool normal;
+    __device__ __forceinline__ explicit Divisor(T a_) : a(a_), r(rcp_steps(a_)), normal(rcp_normal(a_)) {}
+    __device__ __forceinline__ T operator()(T x) const { return normal ? x * r : x / a; }
+};
+template <typename T>
+__device__ __forceinline__ T rcp_nr(T a) {
+    return rcp_normal(a) ? rcp_steps(a) : (T)1 / a;
 }
 
 __device__ __forceinline__ double dec(double s, double, double) { return s; }
