@@ -22,7 +22,7 @@ SOURCES = ["lbm_vanse.cu", "vanse_warp_solid.cu", "vanse_warp_jb.cu", "vanse_war
            "lbm_vanse3d.cu"]
 HEADERS = ["vanse_common.cuh", "vanse_step.cuh", "vanse_aux.cuh", "vanse_pair.cuh", "vanse_warp.cuh",
            "vanse_tile.cuh", "step_rules.h",
-           "vanse_batch.cuh", "mms_force.cuh", "vanse_adjoint.cuh"]
+           "vanse_batch.cuh", "mms_force.cuh", "vanse_adjoint.cuh", "adjoint_plan.h"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -20,6 +20,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "adjoint_plan.h"
 #include "lbm_vanse.h"
 #include "step_rules.h"
 #include "vanse_adjoint.cuh"
@@ -2101,7 +2102,7 @@ namespace {
 struct AdjBuffers {
     std::vector<std::pair<double**, long long>> wanted;
     char* base = nullptr;
-    long long bytes = 0;
+    long long bytes = 0, failed = 0;   // wanted; of the last try that the device could not hold
     void* host = nullptr;         // pinned host checkpoints
     long long host_bytes = 0;
     cudaStream_t st = nullptr;
@@ -2110,10 +2111,19 @@ struct AdjBuffers {
         wanted.push_back({p, bytes});
         bytes += (n * (long long)sizeof(double) + 255) / 256 * 256;
     }
-    void allocate() {
-        if (err == cudaSuccess) err = cudaMallocAsync((void**)&base, (size_t)bytes, st);
-        if (err != cudaSuccess) { base = nullptr; return; }
-        for (auto& w : wanted) *w.first = (double*)(base + w.second);
+    // 0, 1 (the device has not that much: everything wanted is forgotten, for a smaller try) or 2
+    int allocate() {
+        err = cudaMallocAsync((void**)&base, (size_t)bytes, st);
+        if (err == cudaSuccess) {
+            for (auto& w : wanted) *w.first = (double*)(base + w.second);
+            return 0;
+        }
+        base = nullptr;
+        if (err != cudaErrorMemoryAllocation) return 2;
+        cudaGetLastError();
+        wanted.clear();
+        failed = std::exchange(bytes, 0);
+        return 1;
     }
     double* get_host(long long n) {
         if (err == cudaSuccess) err = cudaMallocHost(&host, (size_t)n * sizeof(double));
@@ -2127,8 +2137,6 @@ struct AdjBuffers {
         if (host) cudaFreeHost(host);
     }
 };
-
-constexpr long long kAdjKeep = 512LL << 20;   // device bytes of states kept instead of recomputed
 
 struct AdjEvents {
     cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
@@ -2177,44 +2185,41 @@ extern "C" lbm_status lbm_vanse_outlet_momentum_grad(const lbm_vanse_params* p, 
     const int T = a->nsteps, M = a->avg_steps, K = a->checkpoint_every;
     const int nck = (T - 1) / K + 1;
     const bool want_grad = dJdphi != nullptr;
-    // One level (dense_segments = 1): checkpoints and a whole segment of K states on the
-    // device. Otherwise the checkpoints are in pinned host memory, and the device holds as
-    // much as fits kAdjKeep: every state after f(0) (nothing is recomputed), or a whole
-    // segment (every step recomputed once), or else sub-segments of K2 states whose first
-    // ones are kept on the host too while a segment is processed (recomputed twice).
-    // The objective alone keeps nothing.
-    const bool dense = a->dense_segments != 0;
-    auto fits = [&](long long states) { return states * N9 * (long long)sizeof(double) <= kAdjKeep; };
-    const bool keep_all = want_grad && !dense && fits(T - 1);
-    const bool whole = dense || fits(std::min(K, T));   // the device holds whole segments
-    const int K2 = whole ? std::min(K, T) : std::max(1, (int)std::ceil(std::sqrt((double)std::min(K, T))));
-    const int nsub = (std::min(K, T) - 1) / K2 + 1;   // sub-checkpoints per segment
+    const bool dense = a->dense_segments != 0;   // what is kept where: adjoint_plan.h (the objective alone: nothing)
 
     AdjBuffers B;
     B.st = st;
     double *d_phi, *fa, *fb, *iphi, *acc, *ck = nullptr, *seg = nullptr, *lam = nullptr, *lam2 = nullptr, *gphi = nullptr;
     adj::Fields F;
     adj::Adj A;
-    B.want(&d_phi, N);
-    B.want(&fa, N9);
-    B.want(&fb, N9);
-    for (double** q : {&iphi, &F.s, &F.rho, &F.ux, &F.uy, &F.Fx, &F.Fy, &F.drx, &F.dry, &F.Ax, &F.Ay, &F.Dx, &F.Dy})
-        B.want(q, N);
-    B.want(&acc, 1);
-    if (want_grad) {
-        if (dense) B.want(&ck, (long long)nck * N9);
-        B.want(&seg, std::max(1LL, keep_all ? T - 1LL : (long long)K2) * N9);
-        for (double** q : {&lam, &lam2, &A.lm}) B.want(q, N9);
-        for (double** q : {&gphi, &A.lux, &A.luy, &A.lFx, &A.lFy, &A.lrho, &A.ldrx, &A.ldry}) B.want(q, N);
-        B.want(&A.lg, 7 * N);
-    }
-    B.allocate();
+    adj::Plan plan{};
+    auto allocate = [&](const adj::Plan& q) {
+        B.want(&d_phi, N);
+        B.want(&fa, N9);
+        B.want(&fb, N9);
+        for (double** f : {&iphi, &F.s, &F.rho, &F.ux, &F.uy, &F.Fx, &F.Fy, &F.drx, &F.dry, &F.Ax, &F.Ay, &F.Dx, &F.Dy})
+            B.want(f, N);
+        B.want(&acc, 1);
+        if (want_grad) {
+            if (dense) B.want(&ck, q.device_ck * N9);
+            B.want(&seg, q.seg * N9);
+            for (double** f : {&lam, &lam2, &A.lm}) B.want(f, N9);
+            for (double** f : {&gphi, &A.lux, &A.luy, &A.lFx, &A.lFy, &A.lrho, &A.ldrx, &A.ldry}) B.want(f, N);
+            B.want(&A.lg, 7 * N);
+        }
+        const int r = B.allocate();
+        if (r == 0 && want_grad && !dense) ck = B.get_host(q.host_states * N9);
+        return r;
+    };
+    if (want_grad) adj::allocate_plan(plan, dense, T, K, N9 * (long long)sizeof(double), allocate);
+    else allocate(plan);
     F.iphi = iphi;
-    if (want_grad && !dense) ck = B.get_host((keep_all ? 1LL : (long long)nck + (whole ? 0 : nsub)) * N9);
+    const bool keep_all = want_grad && plan.keep == adj::Keep::all && !dense, whole = plan.keep != adj::Keep::subsegment;
+    const int K2 = plan.K2;
     double* ck1 = ck + (long long)nck * N9;   // host: a segment's sub-checkpoints (not whole)
     if (B.err != cudaSuccess)
         return fail(nullptr, B.err == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA,
-                    "adjoint buffers (%lld device bytes, %lld host bytes): %s", B.bytes, B.host_bytes,
+                    "adjoint buffers (%lld device bytes, %lld host bytes): %s", B.base ? B.bytes : B.failed, B.host_bytes,
                     cudaGetErrorString(B.err));
 #define ACK(call)                                                                                              \
     do {                                                                                                       \
