@@ -105,7 +105,9 @@ struct lbm_vanse {
     long long steps = 0;
     // step-kernel launch shape
     int W = 0, H = 0, gridx = 0, gridy = 0;
-    int resident = 1;             // step-kernel CTAs resident on the device
+    // by the rows of phi and force a step stages (step_rows; they take shared memory):
+    // step-kernel CTAs resident on the device, and rows per strip (H is that of one row)
+    int resident[5] = {1, 1, 1, 1, 1}, strip_rows[5] = {0, 0, 0, 0, 0};
     // replayed graph of kGraphSteps steady steps, valid while its key matches
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -253,15 +255,25 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
 }
 
 // The launch rules of step_rules.h on this handle.
-StepShape step_shape(const lbm_vanse* h) {
-    return StepShape{h->prm.nx, h->prm.ny, h->gridx,      h->resident,  h->nsm,
-                     h->kernel, h->sbytes, h->prm.strip_rows, h->has_solid, h->auto_kernel};
+StepShape step_shape(const lbm_vanse* h, int nR = 1) {
+    return StepShape{h->prm.nx, h->prm.ny, h->gridx,          h->resident[nR], h->nsm,
+                     h->kernel, h->sbytes, h->prm.strip_rows, h->has_solid,    h->auto_kernel};
 }
 
+// One height by the rows staged: with force rows FP32 CTAs are 7 per SM instead of 8, and a
+// height that fills one wave of 8 leaves a second wave nearly empty (us a step with a force
+// field, height by its own residency / by that without: 1000 x 700 FP32 20.5 / 30.7, 631 x 1432
+// 24.3 / 38.7, 2000 x 1500 71.8 / 85.6). With solid cells one height for all: their flags are
+// kept by CTA.
 void pick_strip_height(lbm_vanse* h) {
     h->H = strip_height(step_shape(h));
     h->gridy = (h->prm.ny + h->H - 1) / h->H;
+    for (int nR = 1; nR <= 4; ++nR)
+        h->strip_rows[nR] = h->kernel == 5 && !h->has_solid ? strip_height(step_shape(h, nR)) : h->H;
 }
+
+// rows of phi(t), phi(t+1), F^B_x and F^B_y that the next step stages with the populations
+int step_rows(const lbm_vanse* h) { return 1 + (h->unsteady ? 1 : 0) + (h->has_fb ? 2 : 0); }
 
 void pick_tile(lbm_vanse* h) {
     const TileShape t = tile_shape(step_shape(h));
@@ -281,12 +293,12 @@ lbm_status configure(lbm_vanse* h) {
     if constexpr (sizeof(S) == 2) {
         if (h->jbase) CK(h, warp_jb_configure<S>(smax));
     }
-    const size_t s1 = step_smem_bytes<S>(h, 1);
-    int per_sm = 0, nsm = 0;
-    CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, s1));
-    CK(h, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device));
-    h->resident = std::max(1, per_sm * nsm);
-    h->nsm = nsm;
+    CK(h, cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device));
+    for (int nR = 1; nR <= 4; ++nR) {
+        int per_sm = 0;
+        CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, step_smem_bytes<S>(h, nR)));
+        h->resident[nR] = std::max(1, per_sm * h->nsm);
+    }
     pick_strip_height(h);
     if constexpr (!std::is_same<S, double>::value) {
         if (h->auto_kernel && h->kernel == 5 && h->prm.eq_order != 2 && !h->jbase && h->prm.strip_rows == 0) {
@@ -384,15 +396,15 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
     p.ny = h->prm.ny;
     p.P = h->P;
     p.W = h->W;
-    p.H = h->H;
     p.wall_y = h->prm.bc_y == LBM_BC_BOUNCEBACK;
     p.wall_x = h->prm.bc_x == LBM_BC_BOUNCEBACK;
     p.unsteady = h->unsteady;
     p.has_fb = h->has_fb;
     p.model_b = h->prm.model_b;
-    const int nR = 1 + (h->unsteady ? 1 : 0) + (h->has_fb ? 2 : 0);
+    const int nR = step_rows(h);
     const size_t smem = step_smem_bytes<S>(h, nR);
     p.nR = nR;
+    p.H = h->strip_rows[nR];
     p.kappa = (R)h->prm.kappa;
     p.gx = (R)h->gx;
     p.gy = (R)h->gy;
@@ -446,7 +458,7 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
         }
     }
     if (h->kernel == 5) p.pop_map = h->pop_map[src];
-    dim3 grid(h->gridx, h->gridy);
+    dim3 grid(h->gridx, row_blocks(h->prm.ny, p.H));
     if (h->has_solid) return launch_solid_step<S>(h, p, grid, smem, stream, sums != nullptr);
     if (sums) {
         if (!h->sums_configured) {
@@ -498,7 +510,7 @@ lbm_status enqueue_step(lbm_vanse* h, cudaStream_t stream, int src, double* sums
                     // predecessor's last ones otherwise pile up on some SMs (800^2, 1120 of
                     // 1216 resident strips: 16.7 us against 15.8; 1200 x 900 24.6 / 25.3 and
                     // 2048^2 62.8 / 66.6 the other way round)
-                    else if ((long long)h->gridx * h->gridy * 16 >= 15LL * h->resident)
+                    else if ((long long)grid.x * grid.y * 16 >= 15LL * h->resident[nR])
                         CK(h, launch_pdl(vanse_warp_kernel<S, LBMV_WARP_MINB>, grid, dim3(32), smem, stream, p));
                     else vanse_warp_kernel<S, LBMV_WARP_MINB><<<grid, 32, smem, stream>>>(p);
                 }
@@ -1563,11 +1575,11 @@ extern "C" lbm_status lbm_vanse_launch_shape(lbm_vanse_t h, int* threads, int* c
     if (!h) return fail(nullptr, LBM_ERR_ARG, "handle is NULL");
     if (threads) *threads = step_threads(h);
     if (cols) *cols = h->W;
-    if (rows) *rows = h->H;
+    const int nR = step_rows(h);
+    if (rows) *rows = h->strip_rows[nR];
     if (grid_x) *grid_x = h->gridx;
-    if (grid_y) *grid_y = h->gridy;
+    if (grid_y) *grid_y = row_blocks(h->prm.ny, h->strip_rows[nR]);
     if (smem_bytes) {
-        const int nR = 1 + (h->unsteady ? 1 : 0) + (h->has_fb ? 2 : 0);
         size_t s = 0;
         switch (h->prm.storage) {
             case LBM_FP64: s = step_smem_bytes<double>(h, nR); break;
