@@ -40,7 +40,10 @@ inline int row_blocks(int ny, int rows) { return (int)(((long long)ny + rows - 1
 // 1531 x 1024 30.0 / 30.4 / 36.1 / 40, 1800 x 1400 42.4 / 42.1 / 46.3 / 53.7, 2048^2
 // 72.2 / 64.9 / 66.4 / 72.6, 3000 x 2500 119 / 105.7 / 104.2 / 110.1, 4001 x 3001
 // 185.9 / 165.8 / 164.4 / 164.2 (five waves of at least 16 rows, the rule before: 21.5,
-// 36.1, 48.1, 72.9, 110.2, 170.1). With solid cells kernel 5 cuts ten waves of at least 16
+// 36.1, 48.1, 72.9, 110.2, 170.1). Where a wave holds a strip or three of each column, w
+// waves' worth of strips rounded down leave the last one far from full; one strip more is
+// taken if that ends sooner by whole waves (FP32 in us: 100000 x 30 54.4 / 49.6, 100000 x 600
+// 803 / 747, 300000 x 100 392 / 383). With solid cells kernel 5 cuts ten waves of at least 16
 // rows: the CTAs next to a solid take several times as long as the others, and shorter
 // strips shorten the longest CTA. FP64 on kernel 1: march64_us; with solid cells only where
 // 16-row strips are fewer than two per SM and no kernel was asked for (us a step, generic
@@ -71,6 +74,12 @@ inline int strip_height(const StepShape& s) {
         int w = 1;
         while (w < 5 && rows(w) > kWaveRows[w - 1]) ++w;
         H = rows(w);
+        auto row_times = [&](int h) {
+            const long long ctas = (long long)s.gridx * row_blocks(s.ny, h);
+            return (ctas + s.resident - 1) / s.resident * (h + 6);
+        };
+        const int one_more = row_blocks(s.ny, std::max(1, w * s.resident / s.gridx) + 1);
+        if (row_times(one_more) < row_times(H)) H = one_more;
     } else if (s.sbytes == 8 &&
                (!s.solid || (s.auto_kernel && (long long)s.gridx * row_blocks(s.ny, 16) < 2LL * s.nsm))) {
         H = least;

@@ -62,3 +62,16 @@ def test_tiles_up_to_the_last_height_that_fits(rules, nx, sbytes, solid):
     """Narrow lattices that tiles suit keep them up to 8 * 65535 rows and march beyond."""
     assert rules(nx, 8 * GRID_Y, sbytes, solid)[1] == 8
     assert rules(nx, 8 * GRID_Y + 1, sbytes, solid)[1] == 0
+
+
+@pytest.mark.parametrize("nx,ny", [(80000, 100), (100000, 30), (100000, 600), (150000, 200), (300000, 100), (72961, 67),
+                                   (4096, 4096), (1200, 900), (800, 800)])
+def test_wide_lattices_do_not_leave_a_wave_to_a_few_strips(rules, nx, ny):
+    """By whole waves of H + 6 rows the height is no worse than five waves of 16 rows and more."""
+    cols, resident = -(-nx // 60), 152 * 8
+
+    def row_times(H):
+        return -(-(cols * -(-ny // H)) // resident) * (H + 6)
+
+    generic = min(ny, max(16, -(-ny // max(1, -(-5 * resident // cols)))))
+    assert row_times(rules(nx, ny, 4, kernel=5)[0]) <= row_times(generic)
