@@ -257,7 +257,8 @@ const void* step_kernel_ptr(const lbm_vanse* h) {
 // The launch rules of step_rules.h on this handle.
 StepShape step_shape(const lbm_vanse* h, int nR = 1) {
     return StepShape{h->prm.nx, h->prm.ny, h->gridx,          h->resident[nR], h->nsm,
-                     h->kernel, h->sbytes, h->prm.strip_rows, h->has_solid,    h->auto_kernel};
+                     h->kernel, h->sbytes, h->prm.strip_rows, h->has_solid,    h->auto_kernel,
+                     h->prm.bc_y == LBM_BC_BOUNCEBACK};
 }
 
 // One height by the rows staged: with force rows FP32 CTAs are 7 per SM instead of 8, and a

@@ -23,6 +23,7 @@ struct StepShape {
     int strip_rows;    // rows asked for, 0 = automatic
     bool solid;        // lattice with solid cells
     bool auto_kernel;  // created without asking for a kernel
+    bool wall_y;       // walls in y
 };
 
 struct TileShape {
@@ -54,11 +55,12 @@ inline int row_blocks(int ny, int rows) { return (int)(((long long)ny + rows - 1
 // march64_us: a CTA (128 threads) keeps an SM's FP64 pipe 5/6 busy by itself, 7.8 us a row,
 // and two on an SM take 13 us a row; a strip of H rows steps through about H + 4. FP64
 // step in us, H = 12 / 16 / 24 / 48: 1024 x 768 380 / 472 / 365 / 406, 2000 x 1500 1317 /
-// 1400 / 1383 / 1392.
+// 1400 / 1383 / 1392. A strip between two walls has no halo rows to work on and steps through
+// about H + 2 (36000 x 8 130 us at 8 rows, where tiles of 4 take 145; 60000 x 20 554 / 610).
 inline double march64_us(const StepShape& s, int H) {
     const long long ctas = (long long)s.gridx * row_blocks(s.ny, H), slots = 2LL * s.nsm;
     const long long rem = ctas % slots;
-    return (H + 4) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= s.nsm ? 7.8 : 13.0)));
+    return (H + (s.wall_y && H >= s.ny ? 2 : 4)) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= s.nsm ? 7.8 : 13.0)));
 }
 
 inline int strip_height(const StepShape& s) {

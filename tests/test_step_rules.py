@@ -12,8 +12,9 @@ GRID_Y = 65535
 SHIM = r"""
 #include "step_rules.h"
 extern "C" void rules(int nx, int ny, int gridx, int resident, int nsm, int kernel, int sbytes, int strip_rows,
-                      int solid, int auto_kernel, int* out) {
-    const lbmv::StepShape s{nx, ny, gridx, resident, nsm, kernel, sbytes, strip_rows, solid != 0, auto_kernel != 0};
+                      int solid, int auto_kernel, int wall, int* out) {
+    const lbmv::StepShape s{nx,         ny,         gridx,            resident, nsm, kernel, sbytes,
+                            strip_rows, solid != 0, auto_kernel != 0, wall != 0};
     out[0] = lbmv::strip_height(s);
     const lbmv::TileShape t = lbmv::tile_shape(s);
     out[1] = sbytes == 8 ? lbmv::tile64_rows(s, out[0]) : t.rows;
@@ -31,11 +32,12 @@ def rules(tmp_path_factory):
                    check=True)
     fn = ctypes.CDLL(lib).rules
 
-    def call(nx, ny, sbytes, solid=False, strip_rows=0, kernel=0):
+    def call(nx, ny, sbytes, solid=False, strip_rows=0, kernel=0, wall=False):
         k = kernel or (1 if sbytes == 8 else 5)
         cols, per_sm = (60, 8) if k == 5 else (124, 2)
         out = (ctypes.c_int * 3)()
-        fn(nx, ny, -(-nx // cols), 152 * per_sm, 152, k, sbytes, strip_rows, int(solid), int(kernel == 0), out)
+        fn(nx, ny, -(-nx // cols), 152 * per_sm, 152, k, sbytes, strip_rows, int(solid), int(kernel == 0), int(wall),
+           out)
         return tuple(out)
 
     return call
@@ -75,3 +77,8 @@ def test_wide_lattices_do_not_leave_a_wave_to_a_few_strips(rules, nx, ny):
 
     generic = min(ny, max(16, -(-ny // max(1, -(-5 * resident // cols)))))
     assert row_times(rules(nx, ny, 4, kernel=5)[0]) <= row_times(generic)
+
+
+@pytest.mark.parametrize("nx,ny", [(30000, 5), (36000, 8)])
+def test_low_walled_fp64_lattices_march_in_one_strip(rules, nx, ny):
+    assert rules(nx, ny, 8, wall=True)[:2] == (ny, 0)
