@@ -223,12 +223,6 @@ size_t step_smem_max(const lbm_vanse* h) {
     return (h->kernel >= 2 && h->kernel <= 5) ? b : b + (h->has_solid ? 0 : StepLayout<S, R, kThreads>::solid_bytes());
 }
 
-// a tile kernel runs the lattice's plain steps (the step sums and the moving wall stay
-// with kernel 5, and those, the moving wall and solid cells in FP64 with kernel 1)
-bool runs_tile(const lbm_vanse* h) {
-    return h->tile_rows > 0 && !h->nee_top && !(h->has_solid && h->prm.storage == LBM_FP64);
-}
-
 int step_threads(const lbm_vanse* h) {
     if (h->kernel == 5) return 32;
     return h->kernel >= 2 ? kPairT[h->kernel - 2] : kThreads;
@@ -271,6 +265,14 @@ void pick_strip_height(lbm_vanse* h) {
     h->gridy = (h->prm.ny + h->H - 1) / h->H;
     for (int nR = 1; nR <= 4; ++nR)
         h->strip_rows[nR] = h->kernel == 5 && !h->has_solid ? strip_height(step_shape(h, nR)) : h->H;
+}
+
+// a tile kernel runs the lattice's plain steps (the step sums and the moving wall stay
+// with kernel 5, and those, the moving wall and solid cells in FP64 with kernel 1)
+bool runs_tile(const lbm_vanse* h) {
+    if (h->tile_rows == 0 || h->nee_top) return false;
+    if (!h->has_solid) return true;
+    return h->prm.storage != LBM_FP64 && solid_tiles_pay(step_shape(h), h->unsteady || h->has_fb || h->has_drag);
 }
 
 // rows of phi(t), phi(t+1), F^B_x and F^B_y that the next step stages with the populations

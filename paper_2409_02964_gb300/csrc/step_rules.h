@@ -117,6 +117,14 @@ inline TileShape tile_shape(const StepShape& s) {
     return TileShape{rows, ctas(4) > 2LL * s.nsm};
 }
 
+// Whether a step of a lattice with solid cells that may run as tiles does: a step with a force
+// field, drag or a moving void fraction (general) takes the longer forms in every tile, while
+// most marching strips gain nothing from their absence, so the line lies lower: 3 M cells (us a
+// step, tiles / marching, one block of solid cells, force field: FP32 1800 x 1600 118.5 / 117.0,
+// 2000 x 1900 156 / 148, 2100^2 177 / 160, BF16 2000 x 1500 126 / 125, 2000 x 1900 158 / 144;
+// scattered ones as well FP32 2000 x 1900 289 / 315, 2100^2 moving 332 / 304).
+inline bool solid_tiles_pay(const StepShape& s, bool general) { return !general || (double)s.nx * s.ny <= 3.0e6; }
+
 // The FP64 tile kernel instead of kernel 1 where it is quicker: rows per CTA by the FP64
 // pipe time of the busiest SM, CTAs per SM times kUs[R] (measured on 2000 x 1500; the same
 // figure predicts every size within 10 %). FP64 step in us, tiles / kernel 1 at 16 rows:
