@@ -12,7 +12,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <functional>
 #include <map>
 #include <numeric>
 #include <string>
@@ -1690,33 +1689,37 @@ void batch_strips(int ny, int H, int* strips, int* rows) {
 // schedule no longer matters: the work per CTA plus one unit. us per step, this rule / 24 /
 // 48 / 96 rows: 24 lattices of 10.96 M cells FP32 188 / 203 / 196 / 185, 7 of 2.3 M 53 / 63
 // / 63 / 99, 40 of 12.6 M 202 / 232 / 213 / 202, 40 of 17.0 M BF16 267 / 296 / 274 / 278.
+// Lattices of one height are taken together, so that thousands of them cost no more than the
+// heights they have (creating 2000 lattices of 20 to 40 rows: 1.8 ms of this rule one by one,
+// 0.08 together).
 int batch_rows(const lbm_vanse_batch* b) {
+    std::map<int, long long> columns;   // by height: columns of units
+    for (const BatchLattice& L : b->desc) columns[L.ny] += L.tiles_x;
     int best = 48;
     double best_cost = 0;
     for (int H = 12; H <= 192; H += H < 64 ? 4 : 16) {
-        std::vector<std::pair<int, long long>> kinds;   // (row times, units)
+        std::vector<long long> of_rows(H + 1, 0);   // units of each height
         double sum = 0;
         long long units = 0;
-        for (const BatchLattice& L : b->desc) {
+        for (const auto& [ny, cols] : columns) {
             int strips, rows;
-            batch_strips(L.ny, H, &strips, &rows);
-            kinds.push_back({rows + 6, (long long)L.tiles_x * strips});
-            sum += (double)(rows + 6) * L.tiles_x * strips;
-            units += (long long)L.tiles_x * strips;
+            batch_strips(ny, H, &strips, &rows);
+            of_rows[rows] += cols * strips;
+            sum += (double)(rows + 6) * cols * strips;
+            units += cols * strips;
         }
         double cost;
         if (units > 12LL * b->grid) {
             cost = sum / b->grid + H + 6;
         } else {
-            std::sort(kinds.begin(), kinds.end(), std::greater<>());
             // CTAs by the time they fall free (whole groups of them take units of one height)
             std::map<int, long long> free_at{{0, b->grid}};
             int end = 0;
-            for (auto& k : kinds)
-                for (long long left = k.second; left > 0;) {
+            for (int rows = H; rows > 0; --rows)
+                for (long long left = of_rows[rows]; left > 0;) {
                     const auto first = free_at.begin();
                     const long long m = std::min(left, first->second);
-                    const int t = first->first + k.first;
+                    const int t = first->first + rows + 6;
                     if ((first->second -= m) == 0) free_at.erase(first);
                     free_at[t] += m;
                     end = std::max(end, t);
