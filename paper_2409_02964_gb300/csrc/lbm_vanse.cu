@@ -1971,8 +1971,11 @@ extern "C" lbm_status lbm_vanse_batch_create(const lbm_vanse_batch_lattice* latt
     int nmax = 0;
     for (auto& q : b->lat) nmax = std::max(nmax, q.n);
     // one copy a thread where that is not many CTAs (in seven rounds of 32 CTAs per lattice the
-    // refresh took a tenth of the step: 24 lattices 192 / 184 us, 7 lattices 51.6 / 45.8)
-    b->ghost_blocks = (int)std::min<long long>((9LL * nmax * 2 * kGhost + 255) / 256, std::max(32, 4096 / count));
+    // refresh took a tenth of the step: 24 lattices 192 / 184 us, 7 lattices 51.6 / 45.8), and
+    // about 16 thousand CTAs in all: each counts itself off at the end (2000 lattices of 20 to 40
+    // rows, 9 CTAs each: 128 us a step, 5 each: 122; 8000 of 16 to 24: 320 / 294)
+    const long long full = (9LL * nmax * 2 * kGhost + 255) / 256, per_thread = (full * count + 16383) / 16384;
+    b->ghost_blocks = (int)std::min<long long>((full + per_thread - 1) / per_thread, std::max(32, 4096 / count));
     if (st == LBM_OK) {
         for (int i = 0; i < count; ++i) {
             const size_t bytes = ((size_t)9 * b->desc[i].plane * b->sbytes + 255) / 256 * 256;
