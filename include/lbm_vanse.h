@@ -315,9 +315,10 @@ lbm_status lbm_vanse_batch_step(lbm_vanse_batch_t b, int nsteps);
  * a lone lattice would be (about five waves of resident CTAs, >= 16 rows). */
 lbm_status lbm_vanse_batch_step_each(lbm_vanse_batch_t b, int nsteps);
 
-/* Time trial_steps steps for each work-unit height of {16, 24, 32, 48, 64, 96, 128,
- * 192, 256}, keep the fastest, write it to *rows_out (may be NULL) and
- * re-initialise the batch (t = 0). */
+/* Time trial_steps steps for the work-unit height the batch has (automatic, or
+ * strip_rows) and for each of {16, 24, 32, 48, 64, 96, 128, 192, 256}, keep the fastest
+ * and re-initialise the batch (t = 0). *rows_out (may be NULL) receives the fastest of
+ * the listed heights; the batch keeps its own where that is faster than all of them. */
 lbm_status lbm_vanse_batch_autotune(lbm_vanse_batch_t b, int trial_steps, int* rows_out);
 
 /* Eq. (26) sums for lattice index at the current step against its manufactured

@@ -74,6 +74,8 @@ class Batch:
         self._call("lbm_vanse_batch_step_each", int(nsteps))
 
     def autotune(self, trial_steps: int = 20) -> int:
+        """The fastest of the listed unit heights (lbm_vanse_batch_autotune); the batch keeps
+        the height it has where that is faster than all of them."""
         rows = ctypes.c_int()
         self._call("lbm_vanse_batch_autotune", int(trial_steps), ctypes.byref(rows))
         return rows.value
