@@ -608,8 +608,9 @@ template <typename S>
 lbm_status run_get(lbm_vanse* h, double* out) {
     using R = typename Prec<S>::R;
     const long long n = (long long)h->prm.nx * h->prm.ny;
-    get_pop_kernel<S, R><<<aux_blocks(n), kAuxThreads, 0, h->stream>>>((const S*)h->f[h->cur], (const R*)h->phi, out,
-                                                                       make_lattice<double>(h));
+    const Lattice<double> L = make_lattice<double>(h);
+    const auto kernel = L.wall_x || L.has_solid || L.jbase ? get_pop_kernel<S, R, true> : get_pop_kernel<S, R, false>;
+    kernel<<<aux_blocks(n), kAuxThreads, 0, h->stream>>>((const S*)h->f[h->cur], (const R*)h->phi, out, L);
     CK(h, cudaGetLastError());
     return LBM_OK;
 }

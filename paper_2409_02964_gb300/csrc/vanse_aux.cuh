@@ -373,7 +373,9 @@ __global__ void init_kernel(S* __restrict__ buf, const R* __restrict__ phi, cons
 // FP64 (L: the lattice's Lattice<double>): a stored deviation d reads back as
 // d / scale + f^rest with f^rest in FP64, so the value carries no rounding at the
 // scale of f, and writing it back returns d.
-template <typename S, typename R>
+// GENERAL: a lattice with x walls, solid cells or the momentum base, none of whose cells is
+// plain (the plain path beside theirs made their FP64 read-back a tenth slower).
+template <typename S, typename R, bool GENERAL>
 __global__ void get_pop_kernel(const S* __restrict__ buf, const R* __restrict__ phi, double* __restrict__ out,
                                const Lattice<double> L) {
     const long long n = (long long)L.nx * L.ny;
@@ -381,7 +383,7 @@ __global__ void get_pop_kernel(const S* __restrict__ buf, const R* __restrict__ 
         int x, y;
         cell_xy(k, L.nx, x, y);
         double f[9];
-        if (plain_cell(L, y)) {
+        if (!GENERAL && plain_cell(L, y)) {
             pull_stored(buf, L, x, y, f);
             const double r0 = L.rest.r0(widen(phi[cell_off(L.P, x, y)]));
             if (Prec<S>::kDev) {
