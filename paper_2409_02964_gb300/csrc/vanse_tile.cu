@@ -35,8 +35,6 @@ template cudaError_t tile_launch<__nv_bfloat16>(const StepParams<float>&, int, b
 // One FP64 step; see the comment at TileCtx64.
 __global__ void __launch_bounds__(32 * (kTile64Rows + 4), 1) vanse_tile64_kernel(const __grid_constant__ StepParams<double> p) {
     extern __shared__ __align__(16) double tile64_smem[];
-    pdl_wait();
-    pdl_next();
     const int lane = threadIdx.x, w = threadIdx.y, nw = blockDim.y;
     const int x0 = blockIdx.x * kTile64Cols, y0 = blockIdx.y * p.H, y1 = min(y0 + p.H, p.ny);
     const TileCtx64 c{p, x0 - 2 + lane};
