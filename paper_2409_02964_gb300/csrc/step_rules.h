@@ -55,12 +55,15 @@ inline int row_blocks(int ny, int rows) { return (int)(((long long)ny + rows - 1
 // march64_us: a CTA (128 threads) keeps an SM's FP64 pipe 5/6 busy by itself, 7.8 us a row,
 // and two on an SM take 13 us a row; a strip of H rows steps through about H + 4. FP64
 // step in us, H = 12 / 16 / 24 / 48: 1024 x 768 380 / 472 / 365 / 406, 2000 x 1500 1317 /
-// 1400 / 1383 / 1392. A strip between two walls has no halo rows to work on and steps through
-// about H + 2 (36000 x 8 130 us at 8 rows, where tiles of 4 take 145; 60000 x 20 554 / 610).
+// 1400 / 1383 / 1392. A strip of all rows has fewer halo rows to work on, H + 3 or, between
+// walls, H + 2 (36000 x 8: 136 and 123 us at 8 rows, where tiles of 4 take 151 and 144). Beyond
+// two CTAs of each row per SM the waves of strips of unequal height overlap and the model no
+// longer holds: five waves of at least 16 rows (60000 x 20 533 us, tiles 621; walled 524, one
+// strip 585).
 inline double march64_us(const StepShape& s, int H) {
     const long long ctas = (long long)s.gridx * row_blocks(s.ny, H), slots = 2LL * s.nsm;
     const long long rem = ctas % slots;
-    return (H + (s.wall_y && H >= s.ny ? 2 : 4)) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= s.nsm ? 7.8 : 13.0)));
+    return (H + (H < s.ny ? 4 : (s.wall_y ? 2 : 3))) * (13.0 * (ctas / slots) + (rem == 0 ? 0.0 : (rem <= s.nsm ? 7.8 : 13.0)));
 }
 
 inline int strip_height(const StepShape& s) {
@@ -82,7 +85,7 @@ inline int strip_height(const StepShape& s) {
         };
         const int one_more = row_blocks(s.ny, std::max(1, w * s.resident / s.gridx) + 1);
         if (row_times(one_more) < row_times(H)) H = one_more;
-    } else if (s.sbytes == 8 &&
+    } else if (s.sbytes == 8 && s.gridx <= 2 * s.nsm &&
                (!s.solid || (s.auto_kernel && (long long)s.gridx * row_blocks(s.ny, 16) < 2LL * s.nsm))) {
         H = least;
         for (int k = least + 1; k <= std::min(s.ny, std::max(128, least)); ++k)
@@ -132,6 +135,7 @@ inline bool solid_tiles_pay(const StepShape& s, bool general) { return !general 
 // 246 (R = 8); 1024 x 768 398 / 365 at 24 rows.
 inline int tile64_rows(const StepShape& s, int march_rows) {
     static const struct { int rows; double us; } kUs[] = {{1, 4.0}, {2, 5.8}, {3, 7.2}, {4, 8.7}, {6, 13.2}, {8, 16.6}};
+    if (s.gridx > 2 * s.nsm && march_rows < s.ny) return 0;
     double best = march64_us(s, march_rows);
     int rows = 0;
     for (const auto& k : kUs) {

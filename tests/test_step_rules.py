@@ -79,6 +79,7 @@ def test_wide_lattices_do_not_leave_a_wave_to_a_few_strips(rules, nx, ny):
     assert row_times(rules(nx, ny, 4, kernel=5)[0]) <= row_times(generic)
 
 
-@pytest.mark.parametrize("nx,ny", [(30000, 5), (36000, 8)])
-def test_low_walled_fp64_lattices_march_in_one_strip(rules, nx, ny):
-    assert rules(nx, ny, 8, wall=True)[:2] == (ny, 0)
+@pytest.mark.parametrize("wall", [False, True])
+@pytest.mark.parametrize("nx,ny,rows", [(30000, 5, 5), (36000, 8, 8), (60000, 20, 16)])
+def test_low_wide_fp64_lattices_march(rules, nx, ny, rows, wall):
+    assert rules(nx, ny, 8, wall=wall)[:2] == (rows, 0)
