@@ -84,31 +84,54 @@ __global__ void ghost_fill_kernel(S* __restrict__ buf, long long plane, int nx, 
     if (blockIdx.x == 0 && threadIdx.x == 0) *step_next = *step_ctr + 1u;
 }
 
-// Solid-cell tiles of the one-warp kernel: per CTA (its 60 columns x0 .., its strip's
-// rows y0 .. y1-1), 1 when the void fraction phi(t) or phi(t+1) is 0 anywhere in what
-// the CTA stages: rows y0-3 .. y1+2 (past a y wall none, periodic rows wrapped) and
-// columns x0-3 .. x0+63 that lie within the lattice or its ghost columns (the columns
-// beyond hold no value a written cell reads). One CTA per tile.
+// Solid-cell flags of the step kernels: per CTA (its 60 columns x0 .., its rows y0 .. y1-1), 1
+// when the void fraction phi(t) or phi(t+1) is 0 anywhere in what the CTA reads: rows y0-3 ..
+// y1+2 (past a y wall none, periodic rows wrapped) and columns x0-3 .. x0+63 that lie within the
+// lattice or its ghost columns (the columns beyond hold no value a written cell reads).
+//
+// First by rows, which reads phi once whatever the kernels' heights: rows[y * gridx + bx] for one
+// row and the columns of one CTA; a warp each.
 template <typename R>
-__global__ void solid_tiles_kernel(const R* __restrict__ phi, const R* __restrict__ phin,
-                                   unsigned char* __restrict__ tiles, int nx, int ny, int P, int W, int H,
-                                   int wall_y) {
-    const int x0 = blockIdx.x * W, y0 = blockIdx.y * H, y1 = min(y0 + H, ny);
-    const int xlo = x0 - kGhost, xhi = min(x0 + 64, nx + kGhost);
-    const int ncol = xhi - xlo, nrow = (y1 + 2) - (y0 - 3) + 1;
-    int found = 0;
-    for (int k = threadIdx.x; k < nrow * ncol; k += blockDim.x) {
-        int y = y0 - 3 + k / ncol;
-        const int x = xlo + k % ncol;
-        if (y < 0 || y >= ny) {
-            if (wall_y) continue;
-            y = ((y % ny) + ny) % ny;
+__global__ void solid_rows_kernel(const R* __restrict__ phi, const R* __restrict__ phin,
+                                  unsigned char* __restrict__ rows, int nx, int ny, int P, int W, int gridx) {
+    const int lane = threadIdx.x & 31;
+    const unsigned n = (unsigned)ny * (unsigned)gridx, step = gridDim.x * (blockDim.x >> 5);
+    for (unsigned k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n; k += step) {
+        const unsigned y = k / (unsigned)gridx;
+        const int x0 = (int)(k - y * (unsigned)gridx) * W, xhi = min(x0 + 64, nx + kGhost);
+        bool found = false;
+        for (int x = x0 - kGhost + lane; x < xhi; x += 32) {
+            const long long o = cell_off(P, x, (int)y);
+            found = found || phi[o] == (R)0 || (phin && phin[o] == (R)0);
         }
-        const long long o = (long long)y * P + kPadCols + x;
-        if (phi[o] == (R)0 || (phin && phin[o] == (R)0)) found = 1;
+        found = __any_sync(0xffffffffu, found);
+        if (lane == 0) rows[k] = (unsigned char)found;
     }
-    found = __syncthreads_or(found);
-    if (threadIdx.x == 0) tiles[blockIdx.y * gridDim.x + blockIdx.x] = (unsigned char)(found != 0);
+}
+
+// Then by CTA, for the marching kernel (strips of H rows, and its two order counters cleared)
+// and for the tile kernel (TH rows; 0: none). One thread per CTA of theirs.
+__global__ void solid_tiles_kernel(const unsigned char* __restrict__ rows, unsigned char* __restrict__ march, int H,
+                                   int* __restrict__ counters, unsigned char* __restrict__ tiles, int TH, int ny,
+                                   int gridx, int wall_y) {
+    const int n1 = gridx * ((ny + H - 1) / H), n2 = TH > 0 ? gridx * ((ny + TH - 1) / TH) : 0;
+    const int first = blockIdx.x * blockDim.x + threadIdx.x;
+    if (first < 2) counters[first] = 0;
+    for (int k = first; k < n1 + n2; k += gridDim.x * blockDim.x) {
+        const bool m = k < n1;
+        const int t = m ? k : k - n1, h = m ? H : TH, by = t / gridx, bx = t - by * gridx, y0 = by * h;
+        const int end = min(y0 + h, ny) + 2;
+        bool found = false;
+        for (int r = y0 - 3; r <= end; ++r) {
+            int y = r;
+            if (y < 0 || y >= ny) {
+                if (wall_y) continue;
+                y = ((y % ny) + ny) % ny;
+            }
+            found = found || rows[(unsigned)y * (unsigned)gridx + (unsigned)bx] != 0;
+        }
+        (m ? march : tiles)[t] = (unsigned char)found;
+    }
 }
 
 // The launch order of the tiles: those with solid cells first (their CTAs take the
