@@ -423,9 +423,9 @@ def adjoint_run(n: int = 1024, nsteps: int = 4000, avg: int = 100, ckpt: int = 2
         J, g, st = P.outlet_momentum(phi, ch)
         fwd_s, bwd_s = st["forward_ms"] / 1e3, st["backward_ms"] / 1e3
         # FP64 flops per cell: a forward step 263; a backward step with its segment
-        # recompute 632 (ncu instruction counts of the adjoint kernels); the two-level
+        # recompute 672 (ncu instruction counts of the adjoint kernels); the two-level
         # scheme recomputes every step once more (263)
-        flops = 263.0 + 632.0 + (0.0 if dense else 263.0)
+        flops = 263.0 + 672.0 + (0.0 if dense else 263.0)
         achieved = flops * lups / (fwd_s + bwd_s) / 1e12
         out[name] = {"J": J, "max_abs_grad": float(g.abs().max()),
                      "forward_s": round(fwd_s, 3), "backward_s": round(bwd_s, 3),

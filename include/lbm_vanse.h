@@ -78,8 +78,9 @@ typedef struct {
     int strip_rows;              /* rows per CTA strip of the step kernel; 0 = automatic */
     int eager;                   /* 1 = launch each step on its own; 0 = replay runs of steady
                                     steps as a captured CUDA graph (default) */
-    int kernel;                  /* step-kernel variant: 0 = automatic (kernel 5, or its phases on
-                                    tiles for small lattices and solid cells; 1 for FP64 and x walls); 1 = one column per thread
+    int kernel;                  /* step-kernel variant: 0 = automatic (5; 1 for FP64 and x walls;
+                                    either one's phases on tiles where that is quicker, see
+                                    lbm_vanse_launch_shape); 1 = one column per thread
                                     (any storage); 2, 3, 4 = two columns per thread on packed FP32
                                     pairs with 64 / 96 / 128-thread CTAs; 5 = one warp per CTA,
                                     two columns per lane (2..5: not FP64) */
@@ -355,7 +356,8 @@ void lbm_vanse_batch_destroy(lbm_vanse_batch_t b);
  * a few fields in all; every step is recomputed twice in the backward pass). Where a
  * whole segment of K states takes at most 512 MiB the device holds that (one
  * recomputation), and where all nsteps states do, it keeps them from the forward pass
- * (none; the host then holds f(0) alone). With
+ * (none; the host then holds f(0) alone); less of the three where the device does not
+ * have the memory. With
  * dense_segments = 1 the checkpoints and a whole segment of K states stay on the
  * device (one recomputation, K + T/K population arrays). Both give bit-identical
  * results. Everything runs in FP64 on the stream given, whatever p->storage says.
@@ -431,8 +433,10 @@ double lbm_vanse_bytes_per_cell(lbm_vanse_t h);
 
 /* Launch shape of the lattice's marching step kernel: threads per CTA, output columns
  * per CTA, rows per strip, CTAs in x and y, dynamic shared memory bytes. Any may be NULL.
- * (With kernel = 0, plain steps of small lattices and of lattices with solid cells run as
- * tiles of 60 columns by 4 or 8 rows instead, one warp per row.) */
+ * (With kernel = 0, plain steps of small lattices run as tiles instead, one warp per row:
+ * 60 columns by 4 or 8 rows, in FP64 28 columns by 1 to 8; so do those of FP32 / FP16 / BF16
+ * lattices with solid cells up to 4.5 M cells, 4 M in 16 bits, 3 M for steps with a force
+ * field, drag or a pending phi(t+1).) */
 lbm_status lbm_vanse_launch_shape(lbm_vanse_t h, int* threads, int* cols, int* rows, int* grid_x,
                                   int* grid_y, int* smem_bytes);
 

@@ -29,7 +29,7 @@ namespace lbmv {
 // the L1 path on the others: 12.4 warp instructions a cell against the marching kernel's 8.
 // FP32 step, this kernel / the marching kernel at 16 rows, one GB300: 64^2 4.1 / 16.3 us
 // (R = 4), 256^2 5.0 / 18.3, 512^2 9.7 / 20.2 (R = 8); with solid cells 130 x 71 6.3 / 65,
-// 512^2 13.9 / 77, 1531 x 1024 53 / 108, 4096^2 490 / 572. Stepped one row at a time the
+// 512^2 13.9 / 77, 1531 x 1024 53 / 108. Stepped one row at a time the
 // marching kernel pays 0.9 us per row, six of them before the first output row.
 constexpr int kTileWarps[2] = {8, 12};
 constexpr int kTileMaxRows = 8;
@@ -197,9 +197,10 @@ cudaError_t tile_launch(const StepParams<float>& p, int gridx, bool solid, bool 
 // The FP64 step on tiles of 28 columns x R rows: one warp per row, one column per lane, the
 // phases of vanse_step.cuh (full populations, FP64 arithmetic), on lattices without x walls,
 // solid cells, a moving wall or the App. B equilibrium. Same split as above. Bound by the
-// FP64 pipe (2 lanes a cycle and SM): R = 8 is 2180 FP64 warp operations, 16.8 us at that
-// rate against 16.6 measured, so the busiest SM's CTAs are the step's time and R follows
-// from that (pick_tile64). 64^2: 137 us (marching, 16 rows) -> 9.6 us.
+// FP64 pipe (2 lanes a cycle and SM): R = 8 is 1660 FP64 warp instructions a CTA, 12.8 us at
+// that rate of the 16.9 that a CTA's share of its SM takes (532 x 512, 8 CTAs per SM), so the
+// busiest SM's CTAs are the step's time and R follows from that (tile64_rows). 64^2: 137 us
+// (marching, 16 rows) -> 9.6 us.
 struct TileCtx64 {
     const StepParams<double>& p;
     int xc;
