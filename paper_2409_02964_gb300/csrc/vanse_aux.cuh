@@ -152,17 +152,17 @@ __global__ void solid_order_kernel(const unsigned char* __restrict__ tiles, int 
 // R); the last CTA hands them to *verdict (pinned host memory) and clears acc for the next
 // call. Block size a multiple of 32.
 //
-// Doubles are judged by their bits: comparisons and the conversion to R run at the FP64 rate (2
+// Doubles are told apart by their bits: comparisons and the conversion to R run at the FP64 rate (2
 // lanes a cycle and SM): setting phi of 4096^2 cells FP32 took 184 us by them, 111 by bits.
 template <typename R>
-__device__ __forceinline__ void judge_phi(double v, bool& ok, bool& zero) {
+__device__ __forceinline__ void classify_phi(double v, bool& ok, bool& zero) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v), minus0 = 1ull << 63;
     ok = ok && (b <= 0x3ff0000000000000ull || b == minus0);   // 0 .. 1 and -0
     // zero in R: as a float everything up to 2^-150, which rounds to even
     zero = zero || (b & ~minus0) <= (sizeof(R) == 4 ? 0x3690000000000000ull : 0ull);
 }
 template <typename R>
-__device__ __forceinline__ void judge_phi(float v, bool& ok, bool& zero) {
+__device__ __forceinline__ void classify_phi(float v, bool& ok, bool& zero) {
     ok = ok && v >= 0.0f && v <= 1.0f;
     zero = zero || v == 0.0f;
 }
@@ -173,7 +173,7 @@ __global__ void check_phi_kernel(const T* __restrict__ phi_t, const T* __restric
     const T* src = blockIdx.y ? phi_next : phi_t;
     bool ok = true, zero = false;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-        judge_phi<R>(src[k], ok, zero);
+        classify_phi<R>(src[k], ok, zero);
     const int bits = (__syncthreads_or(!ok) ? (blockIdx.y ? 2 : 1) : 0) | (__syncthreads_or(zero) ? 4 : 0);
     if (threadIdx.x != 0) return;
     if (bits) atomicOr(acc, bits);
