@@ -2054,7 +2054,8 @@ extern "C" lbm_status lbm_vanse_batch_autotune(lbm_vanse_batch_t b, int trial_st
         const int H = k < 0 ? current : candidates[k];
         lbm_status st = batch_decompose(b, H);
         if (st == LBM_OK) st = lbm_vanse_batch_init(b);
-        if (st == LBM_OK) st = lbm_vanse_batch_step(b, 2);  // warm-up (and graph capture)
+        // warm-up, with the capture of the graph that the timed steps replay
+        if (st == LBM_OK) st = lbm_vanse_batch_step(b, std::max(2, std::min(trial_steps, kBatchGraphSteps)));
         if (st != LBM_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
         BCK(b, cudaEventRecord(e0, b->stream));
         st = lbm_vanse_batch_step(b, trial_steps);
